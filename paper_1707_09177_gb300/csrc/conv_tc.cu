@@ -2,8 +2,9 @@
 // tensor cores (tcgen05): an implicit GEMM whose accumulator lives in tensor
 // memory and whose activation rows are staged by TMA.
 //
-// One CTA owns an x-segment of 128 points of one (field, z) plane and a range
-// of y. Output row y is
+// A column is an x-segment of 128 points of one (field, z) plane with its Y
+// rows; each of the persistent CTAs (one per SM) works through whole columns
+// and an even share of the rows of those left over (seg_at). Output row y is
 //     D_y[128 points][32 out channels] = sum over taps (dz, dy, dx) and 2 halves of
 //         16 input channels of  A_{z+dz-1, y+dy-1, dx}[128][16] * W_{dz,dy,dx}[16][32].
 // The CTA walks the INPUT rows y' instead: one input row (three z planes)
@@ -41,11 +42,21 @@
 // Every mbarrier wait is bounded by %globaltimer; a CTA whose wait runs out
 // sets the error flag, stops issuing work, waits (bounded) for what it has in
 // flight, frees its tensor memory and returns.
+//
+// What bounds it: an MMA of M = 128, N = 96, K = 16 reads 7 KB of shared memory
+// and takes 56 cycles for 48 of tensor work, 1,134 per input row with the runs
+// split at the ring's wrap; a row takes about 1,350. One 256^3 field: 1.27 ms a
+// layer with the MMAs issued by one lane of a divergent branch (80 cycles each,
+// then 500 more per row for its waits and commits), 0.78 ms issued by the
+// converged warp with the next row's barriers looked at in advance. Whole
+// columns as CTAs of a plain grid ran 10.1 waves on 256^3 x 3; the even split
+// of seg_at took a layer there from 3.33 to 3.01 ms, the issue to 2.3.
 
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -133,12 +144,37 @@ __device__ __forceinline__ uint32_t idesc_n(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTM >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc) {
+// One lane of a converged warp; the same lane every time.
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t e;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(e));
+  return e;
+}
+
+// Issued by the elected lane of a converged warp. The warp-uniform operands
+// stay in uniform registers that way; issued inside a divergent branch, each
+// MMA spent 80 cycles moving its descriptors there, more than the 56 it runs.
+__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, 1, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(dtmem), "l"(a), "l"(b), "r"(idesc)
+      "setp.ne.b32 q, %4, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(elected)
+      : "memory");
+}
+
+// The barrier's arrival when every MMA issued so far has completed.
+__device__ __forceinline__ void mma_commit(uint32_t bar, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      ::"r"(bar), "r"(elected)
       : "memory");
 }
 
@@ -161,25 +197,48 @@ struct ConvTcArgs {
   const uint4* Wimg;             // kWBytes: B operands in shared-memory order
   __nv_bfloat16* Hout;
   const __nv_bfloat16* Hmask;    // mode 1
-  int X, Y, Z;
-  int ychunk;                    // y rows per CTA
+  int X, Y, Z, B;
   int mode;                      // 0: ReLU; 1: zero where the mask is not positive
   unsigned long long wait_ns;
   int* flag;                     // set to 1 when a bounded wait runs out
 };
 
-// grid x = (X/128) * Z * (Y/ychunk), grid y = fields; kThreads threads
+// The work of CTA k of G: a column is one (field, z plane, x segment) with its
+// Y rows. The CTAs take whole columns in rounds (columns k, k + G, ..: the
+// columns worked on at one time are neighbours in z and share their input
+// planes in L2), and the rows of the columns left over are split evenly, so no
+// SM idles through a last partial round. Segment j of CTA k; n = 0 past the end.
+struct Seg {
+  int x0, z, b, y0, n;
+};
+__device__ __forceinline__ Seg seg_at(const ConvTcArgs& a, int j) {
+  const int nxs = a.X / kTM, G = gridDim.x, k = blockIdx.x;
+  const int cols = nxs * a.Z * a.B, full = cols / G;
+  Seg s;
+  int col;
+  if (j < full) {
+    col = j * G + k;
+    s.y0 = 0;
+    s.n = a.Y;
+  } else {
+    const long long rows = (long long)(cols - full * G) * a.Y;
+    const long long lo = rows * k / G, hi = rows * (k + 1) / G;
+    const long long st = j == full ? lo : (lo / a.Y + (j - full)) * a.Y;
+    s.y0 = (int)(st % a.Y);
+    s.n = st < hi ? (int)min(hi - st, (long long)(a.Y - s.y0)) : 0;
+    col = full * G + (int)(st / a.Y);
+  }
+  s.x0 = (col % nxs) * kTM;
+  col /= nxs;
+  s.z = col % a.Z;
+  s.b = col / a.Z;
+  return s;
+}
+
+// grid x = persistent CTAs (one per SM at most); kThreads threads
 __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__ CUtensorMap tmap, const ConvTcArgs a) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nxs = a.X / kTM;
-  int r = blockIdx.x;
-  const int xs = r % nxs;
-  r /= nxs;
-  const int z = r % a.Z;
-  const int yc = r / a.Z;
-  const int b = blockIdx.y;
-  const int x0 = xs * kTM, yb = yc * a.ychunk, ny = a.ychunk;
   // barriers: full[kSlots] / empty[kSlots] (input ring slot staged / read by its MMAs),
   // accf[16] (output row's accumulator complete), acce[16] (read back and cleared)
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kBarOff);
@@ -245,26 +304,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const long long plane_rows = (long long)a.Y * a.Z;     // rows per field
-  const int nrows = ny + 2;                              // input rows: y positions yb - 1 .. yb + ny
   auto row_smem = [&](int s, int zi) { return kRowsOff + (s * 3 + zi) * kRow; };
-  // accumulator slot of output row yb + m: consecutive output rows take
+  // accumulator slot of the CTA's m-th output row: consecutive output rows take
   // consecutive slots downwards, so rows y'+1, y', y'-1 are ascending slots
-  auto acc_slot = [&](int m) { return (kAcc * 4096 - m) % kAcc; };
+  auto acc_slot = [&](int m) { return (int)((0u - (unsigned)m) % (unsigned)kAcc); };
   // bounded wait that also gives up when another role has aborted
+  auto test = [&](uint32_t bar, uint32_t parity) -> bool {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return done != 0;
+  };
   auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
     if (a.wait_ns == 0) return false;
-    {
-      // fast path: a phase that has completed costs no timer read
-      uint32_t done;
-      asm volatile(
-          "{\n\t.reg .pred p;\n\t"
-          "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-          "selp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(done)
-          : "r"(bar), "r"(parity)
-          : "memory");
-      if (done) return true;
-    }
+    if (test(bar, parity)) return true;      // a phase that has completed costs no timer read
     // the abort flag and the timer are read every 64 polls only: polling
     // competes with the tensor cores for shared-memory bandwidth
     const uint64_t t0 = gtime();
@@ -292,112 +350,142 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
   };
 
   if (warp == 4) {
-    // ---- producer: input rows i = 0 .. nrows-1 (y position yb - 1 + i) into
-    // slot i % kSlots: per z plane one TMA load of the 128 interior points
-    // (rows kInterior ..), and the two periodic neighbours (rows kInterior - 1
-    // and kInterior + 128) by lanes 0-23, 16 bytes each (plane lane / 8, side
-    // (lane / 4) & 1, chunk lane & 3), loaded one input row ahead so that
-    // their latency overlaps the previous row's staging
+    // ---- producer: the CTA's gi-th input row (row i of its segment: y position
+    // y0 - 1 + i, i = 0 .. n + 1) into slot gi % kSlots: per z plane one TMA load
+    // of the 128 interior points (rows kInterior ..), and the two periodic
+    // neighbours (rows kInterior - 1 and kInterior + 128) by lanes 0-23, 16 bytes
+    // each (plane lane / 8, side (lane / 4) & 1, chunk lane & 3), loaded one input
+    // row ahead so that their latency overlaps the previous row's staging
     const int hzi = lane >> 3, hside = (lane >> 2) & 1, hc = lane & 3;
-    const int hx = hside ? wrapi(x0 + kTM, a.X) : wrapi(x0 - 1, a.X);
-    auto halo_load = [&](int i) -> uint4 {
-      const long long row = (long long)b * plane_rows + (long long)wrapi(z + hzi - 1, a.Z) * a.Y + wrapi(yb - 1 + i, a.Y);
+    auto halo_load = [&](const Seg& g, int i) -> uint4 {
+      const int hx = hside ? wrapi(g.x0 + kTM, a.X) : wrapi(g.x0 - 1, a.X);
+      const long long row = (long long)g.b * plane_rows + (long long)wrapi(g.z + hzi - 1, a.Z) * a.Y + wrapi(g.y0 - 1 + i, a.Y);
       return *reinterpret_cast<const uint4*>(a.Hin + (row * a.X + hx) * kCh + hc * 8);
     };
     uint4 hv = make_uint4(0u, 0u, 0u, 0u);
-    if (lane < 24) hv = halo_load(0);
-    for (int i = 0; i < nrows; ++i) {
-      const int s = i % kSlots;
-      bool ok = true;
-      if (i >= kSlots) ok = wait_warp(empty0 + 8 * s, (uint32_t)(((i / kSlots) - 1) & 1));
-      if (!ok) { *abort_flag = 1; break; }
-      if (lane < 24) {
-        const uint32_t ra = sbase + row_smem(s, hzi) + (hside ? kInterior + kTM : kInterior - 1) * kPt;
-        const uint32_t dst = ra + ((uint32_t)(hc ^ ((ra >> 7) & 3)) << 4);
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(hv.x), "r"(hv.y), "r"(hv.z), "r"(hv.w)
-                     : "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (i + 1 < nrows) hv = halo_load(i + 1);
-      }
-      __syncwarp();
-      if (lane == 0) {
-        const uint32_t bar = full0 + 8 * s;
-        const int yw = wrapi(yb - 1 + i, a.Y);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kTxBytes) : "memory");
-#pragma unroll
-        for (int zi = 0; zi < 3; ++zi) {
-          const int row = (int)((long long)b * plane_rows + (long long)wrapi(z + zi - 1, a.Z) * a.Y + yw);
-          tma_load3(sbase + row_smem(s, zi) + kInterior * kPt, &tmap, 0, x0, row, bar);
+    Seg g = seg_at(a, 0);
+    if (lane < 24 && g.n) hv = halo_load(g, 0);
+    bool ok = true;
+    int gi = 0;
+    for (int j = 0; ok && g.n; ++j) {
+      const Seg next = seg_at(a, j + 1);
+      for (int i = 0; i < g.n + 2; ++i, ++gi) {
+        const int s = gi % kSlots;
+        if (gi >= kSlots) ok = wait_warp(empty0 + 8 * s, (uint32_t)(((gi / kSlots) - 1) & 1));
+        if (!ok) { *abort_flag = 1; break; }
+        if (lane < 24) {
+          const uint32_t ra = sbase + row_smem(s, hzi) + (hside ? kInterior + kTM : kInterior - 1) * kPt;
+          const uint32_t dst = ra + ((uint32_t)(hc ^ ((ra >> 7) & 3)) << 4);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(hv.x), "r"(hv.y), "r"(hv.z), "r"(hv.w)
+                       : "memory");
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          if (i + 1 < g.n + 2) hv = halo_load(g, i + 1);
+          else if (next.n) hv = halo_load(next, 0);
         }
-        *rows_issued = i + 1;
+        __syncwarp();
+        if (lane == 0) {
+          const uint32_t bar = full0 + 8 * s;
+          const int yw = wrapi(g.y0 - 1 + i, a.Y);
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kTxBytes) : "memory");
+#pragma unroll
+          for (int zi = 0; zi < 3; ++zi) {
+            const int row = (int)((long long)g.b * plane_rows + (long long)wrapi(g.z + zi - 1, a.Z) * a.Y + yw);
+            tma_load3(sbase + row_smem(s, zi) + kInterior * kPt, &tmap, 0, g.x0, row, bar);
+          }
+          *rows_issued = gi + 1;
+        }
+        __syncwarp();
       }
-      __syncwarp();
+      g = next;
     }
   } else if (warp == 5) {
-    // ---- MMA issue (lane 0): input row i = y' - (yb - 1) touches output rows
-    // m = i, i - 1, i - 2 (relative to yb) through dy = 0, 1, 2
-    if (lane == 0) {
-      // descriptors of the first A tile (slot 0, dz = dx = kc = 0) and the
-      // first B block (dz = dx = kc = 0, dy = 0)
-      const uint64_t a0 = sdesc_sw64(sbase + kRowsOff + (kInterior - 1) * kPt);
-      const uint64_t b0 = sdesc(sbase, kBBlock / 2, 128);
-      for (int i = 0; i < nrows; ++i) {
-        bool ok = wait(full0 + 8 * (i % kSlots), (uint32_t)((i / kSlots) & 1));
-        if (ok) *rows_ready = i + 1;
-        // output row m = i enters the ring: its slot's previous row (m - 16)
+    // ---- MMA issue (one elected lane of the converged warp): input row i of a
+    // segment (y' = y0 - 1 + i) touches the segment's output rows i, i - 1, i - 2
+    // through dy = 0, 1, 2. The tensor pipe queues few MMAs, so the next row's
+    // barriers are looked at before this row's last ones are issued: with both
+    // phases complete (they nearly always are) the next row follows at once.
+    const uint32_t el = elect_lane();
+    // descriptors of the first A tile (slot 0, dz = dx = kc = 0) and the
+    // first B block (dz = dx = kc = 0, dy = 0)
+    const uint64_t a0 = sdesc_sw64(sbase + kRowsOff + (kInterior - 1) * kPt);
+    const uint64_t b0 = sdesc(sbase, kBBlock / 2, 128);
+    int gi = 0, mo = 0;              // input rows of the CTA so far; its output rows before this segment
+    bool ok = true, full_ok = false, acc_ok = false;   // next row staged / next accumulator free, seen early
+    for (int j = 0; ok; ++j) {
+      const Seg g = seg_at(a, j);
+      if (!g.n) break;
+      for (int i = 0; i < g.n + 2; ++i) {
+        const int sl = gi % kSlots;
+        if (!full_ok) ok = wait_warp(full0 + 8 * sl, (uint32_t)((gi / kSlots) & 1));
+        // output row m enters the ring: its slot's previous row (m - 16)
         // must have been read back and cleared
-        if (ok && i < ny && i >= kAcc) ok = wait(acce0 + 8 * acc_slot(i), (uint32_t)(((i - kAcc) / kAcc) & 1));
+        const int m = mo + i;
+        if (ok && i < g.n && m >= kAcc && !acc_ok)
+          ok = wait_warp(acce0 + 8 * acc_slot(m), (uint32_t)(((m - kAcc) / kAcc) & 1));
         if (!ok) { *abort_flag = 1; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int hi = min(i, ny - 1), lo = max(i - 2, 0);          // output rows in this CTA's range
-        if (hi >= lo) {
-          // runs of consecutive slots: rows hi, hi - 1, .., lo ascend through the slots
-          int m0 = hi, cnt = hi - lo + 1;
-          while (cnt > 0) {
-            const int s0 = acc_slot(m0);
-            const int run = min(cnt, kAcc - s0);
-            const int g0 = i - m0;                                  // tap dy of output row m0
-            const uint32_t dt = tmem + (uint32_t)(s0 * 32);
-            const uint32_t idesc = idesc_n(32 * run);
-            // the 18 MMAs of the run: their descriptors differ from the row's
-            // first ones by compile-time offsets (in 16-byte units of the
-            // start-address field, which stays below 2^14 inside shared
-            // memory), so the issuing thread spends a few instructions per MMA
-            const uint64_t arow = a0 + (uint64_t)((i % kSlots) * (3 * kRow / 16));
-            const uint64_t brow = b0 + (uint64_t)(g0 * (512 / 16));
-#pragma unroll
-            for (int dz = 0; dz < 3; ++dz)
-#pragma unroll
-              for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-                for (int kc = 0; kc < 2; ++kc)
-                  mma_f16(dt, arow + (uint64_t)((dz * kRow + dx * kPt + kc * 32) / 16),
-                          brow + (uint64_t)((((dz * 3 + dx) * 2 + kc) * kBBlock) / 16), idesc);
-            m0 -= run;
-            cnt -= run;
+        const int hi = mo + min(i, g.n - 1), lo = mo + max(i - 2, 0);
+        const uint64_t arow = a0 + (uint64_t)(sl * (3 * kRow / 16));
+        auto look = [&]() {
+          bool f = false, c = false;
+          if (a.wait_ns) {
+            f = test(full0 + 8 * ((gi + 1) % kSlots), (uint32_t)(((gi + 1) / kSlots) & 1));
+            c = i + 1 < g.n && m + 1 >= kAcc &&
+                test(acce0 + 8 * acc_slot(m + 1), (uint32_t)(((m + 1 - kAcc) / kAcc) & 1));
           }
-        }
+          full_ok = __all_sync(0xffffffffu, f);
+          acc_ok = __all_sync(0xffffffffu, c);
+        };
+        // the 18 MMAs of output rows m0, m0 - 1, .. in `run` consecutive slots:
+        // their descriptors differ from the row's first ones by compile-time
+        // offsets (in 16-byte units of the start-address field, which stays
+        // below 2^14 inside shared memory)
+        auto issue = [&](int m0, int run, bool looking) {
+          const uint32_t dt = tmem + (uint32_t)(acc_slot(m0) * 32);
+          const uint32_t idesc = idesc_n(32 * run);
+          const uint64_t brow = b0 + (uint64_t)((m - m0) * (512 / 16));     // tap dy = m - m0 of row m0
+#pragma unroll
+          for (int dz = 0; dz < 3; ++dz)
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+              if (looking && dz == 2 && dx == 1) look();
+#pragma unroll
+              for (int kc = 0; kc < 2; ++kc)
+                mma_f16(dt, arow + (uint64_t)((dz * kRow + dx * kPt + kc * 32) / 16),
+                        brow + (uint64_t)((((dz * 3 + dx) * 2 + kc) * kBBlock) / 16), idesc, el);
+            }
+        };
+        // rows hi, hi - 1, .., lo ascend through the slots; two runs where they wrap around the ring
+        const int cnt = hi - lo + 1, run = min(cnt, kAcc - acc_slot(hi));
+        if (run < cnt) issue(hi, run, false);
+        issue(run < cnt ? hi - run : hi, run < cnt ? cnt - run : cnt, true);
         // the staged row is read by no later MMA
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         empty0 + 8 * (i % kSlots))
-                     : "memory");
+        mma_commit(empty0 + 8 * sl, el);
         // output row i - 2 receives nothing more
-        if (i >= 2 && i - 2 < ny)
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           accf0 + 8 * acc_slot(i - 2))
-                       : "memory");
-        *rows_done = i + 1;
+        if (i >= 2) mma_commit(accf0 + 8 * acc_slot(m - 2), el);
+        ++gi;
       }
+      mo += g.n;
+    }
+    // for the drain of an aborted CTA: rows staged that this warp waited for, rows committed
+    if (lane == 0) {
+      *rows_ready = gi;
+      *rows_done = gi;
     }
     __syncwarp();
   } else {
-    // ---- epilogue warps 0-3: output rows m = 0 .. ny-1
+    // ---- epilogue warps 0-3: the CTA's output rows m = 0, 1, ..
     uint32_t zr[32];
 #pragma unroll
     for (int q = 0; q < 32; ++q) zr[q] = 0u;
-    for (int m = 0; m < ny; ++m) {
+    int m = 0;
+    bool ok = true;
+    for (int j = 0; ok; ++j) {
+     const Seg g = seg_at(a, j);
+     if (!g.n) break;
+     for (int i = 0; i < g.n; ++i, ++m) {
       const int sl = acc_slot(m);
-      const bool ok = wait_warp(accf0 + 8 * sl, (uint32_t)((m / kAcc) & 1));
+      ok = wait_warp(accf0 + 8 * sl, (uint32_t)((m / kAcc) & 1));
       if (!ok) { *abort_flag = 1; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       uint32_t v[32];
@@ -426,8 +514,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acce0 + 8 * sl) : "memory");
-      const int y = yb + m;
-      const long long p = (((long long)b * a.Z + z) * a.Y + y) * a.X + x0 + warp * 32 + lane;
+      const long long p = (((long long)g.b * a.Z + g.z) * a.Y + g.y0 + i) * a.X + g.x0 + warp * 32 + lane;
       uint4* dst = reinterpret_cast<uint4*>(a.Hout + p * kCh);
       uint4 mk[4];
       if (a.mode == 1) {
@@ -450,6 +537,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
         }
         dst[q] = make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
       }
+     }
     }
   }
   __syncthreads();
@@ -521,15 +609,6 @@ cudaError_t conv_tc_pack(const float* W, __nv_bfloat16* img, int transposed, cud
 
 size_t conv_tc_image_bytes() { return (size_t)kWBytes; }
 
-// y rows per CTA: the largest power-of-two divisor of Y (at most Y) that still
-// gives at least two CTAs per SM over the launch, but no fewer than 4 rows.
-static int pick_ychunk(int X, int Y, int Z, int B, int nsm) {
-  const long long cols = (long long)(X / kTM) * Z * B;
-  int yc = Y;
-  while (yc % 2 == 0 && yc / 2 >= 4 && cols * (Y / yc) < 2LL * nsm) yc /= 2;
-  return yc;
-}
-
 cudaError_t conv_tc_forward(const __nv_bfloat16* Hin, const __nv_bfloat16* Wimg, __nv_bfloat16* Hout,
                             const __nv_bfloat16* Hmask, int X, int Y, int Z, int B, int mode, int* flag,
                             unsigned long long wait_ns, cudaStream_t s) {
@@ -562,12 +641,13 @@ cudaError_t conv_tc_forward(const __nv_bfloat16* Hin, const __nv_bfloat16* Wimg,
   a.X = X;
   a.Y = Y;
   a.Z = Z;
-  a.ychunk = pick_ychunk(X, Y, Z, B, nsm);
+  a.B = B;
   a.mode = mode;
   a.wait_ns = wait_ns;
   a.flag = flag;
-  const dim3 grid((unsigned)((X / kTM) * Z * (Y / a.ychunk)), (unsigned)B);
-  k_conv_tc<<<grid, kThreads, kSmemAlloc, s>>>(map, a);
+  // one CTA per SM (its shared memory is the whole SM's); at least 4 rows each
+  const long long rows = (long long)(X / kTM) * Z * B * Y;
+  k_conv_tc<<<(unsigned)std::min<long long>(nsm, std::max<long long>(1, rows / 4)), kThreads, kSmemAlloc, s>>>(map, a);
   return cudaGetLastError();
 }
 
