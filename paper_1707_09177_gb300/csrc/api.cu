@@ -1096,7 +1096,8 @@ ad_status get_cnn(ad_ctx* ctx, const ad_grid* g, int B, bool training, CnnWork**
         (s = cnn_alloc(ctx, cw, (void**)&w.frag3, frag)) != AD_OK ||
         (s = cnn_alloc(ctx, cw, (void**)&w.frag2t, frag)) != AD_OK ||
         (s = cnn_alloc(ctx, cw, (void**)&w.frag3t, frag)) != AD_OK ||
-        (s = cnn_alloc(ctx, cw, (void**)&w.frag4, sizeof(uint2) * 27 * 2 * 32)) != AD_OK ||
+        (s = cnn_alloc(ctx, cw, (void**)&w.frag4, sizeof(uint2) * 2 * 4 * 32)) != AD_OK ||
+        (s = cnn_alloc(ctx, cw, (void**)&w.frag4t, sizeof(uint2) * 180 * 32)) != AD_OK ||
         (s = cnn_alloc(ctx, cw, (void**)&w.H1, act)) != AD_OK ||
         (s = cnn_alloc(ctx, cw, (void**)&w.H2, act)) != AD_OK ||
         (s = cnn_alloc(ctx, cw, (void**)&w.H3, act)) != AD_OK ||

@@ -8,7 +8,7 @@
 // The 32 -> 32 layers are implicit GEMMs on the tensor cores (bf16 inputs,
 // float32 accumulation): for an x-segment of 32 points per warp, the product
 // over K = 27 taps x 32 input channels into N = 32 output channels; the 32 -> 1
-// last layer is the same GEMM with one n8 tile (column 0). The 1 -> 32 first
+// last layer sums over channels first (27 GEMM columns, one per tap), then over taps. The 1 -> 32 first
 // layer runs on the CUDA cores in float32, so the small differences it forms
 // from u_bar are not lost to bfloat16 rounding. The
 // output is scaled by the fixed factor A = (delta/h)^2 = 1/(pi gamma)^2, the
@@ -68,32 +68,29 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t* r, const void* p) {
                : "r"(s));
 }
 
+// a * b + c of both halves of a pair in one instruction, each rounded as fmaf.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(d)
+      : "l"(*reinterpret_cast<const uint64_t*>(&a)), "l"(*reinterpret_cast<const uint64_t*>(&b)),
+        "l"(*reinterpret_cast<const uint64_t*>(&c)));
+  return *reinterpret_cast<float2*>(&d);
+}
+
 // Row of a shared-memory point tile: 32 bf16 channels (64 bytes) + 16 bytes of
 // padding, so the 8-row ldmatrix phases hit distinct banks.
 constexpr int ROWB = 80;
 
-// Copies the x-segment [x0 - 1, x0 + TX + 1) (periodic) of activation row
-// (b, z, y) into `dst` (TX + 2 rows of ROWB bytes), 16 bytes per thread step.
-__device__ __forceinline__ void load_row(unsigned char* dst, const __nv_bfloat16* H, long long rowbase, int X,
-                                         int x0, int TX, int tid, int nthr) {
-  const int n16 = (TX + 2) * 4;
-  for (int i = tid; i < n16; i += nthr) {
-    const int pt = i >> 2, q = i & 3;
-    const int x = wrap(x0 - 1 + pt, X);
-    const uint4 v = *reinterpret_cast<const uint4*>(H + (rowbase + x) * C + q * 8);
-    *reinterpret_cast<uint4*>(dst + pt * ROWB + q * 16) = v;
-  }
-}
-
-// Asynchronous form of load_row for the three rows (b = 0..2) of z offset a:
-// 16-byte cp.async copies into `dst` (3 rows of TX + 2 points, ROWB bytes per
-// point), committed as one group by the caller.
+// Copies the x-segment [x0 - 1, x0 + TX + 1) (periodic) of the `nr` activation
+// rows y - 1 .. y + nr - 2 of z offset a into `dst` (rows of TX + 2 points, ROWB
+// bytes per point): 16-byte cp.async copies, committed as one group.
 __device__ __forceinline__ void stage_rows_async(unsigned char* dst, const __nv_bfloat16* H, long long base, int z,
-                                                 int y, int a, int X, int Y, int Z, int x0, int TX, int tid,
+                                                 int y, int a, int nr, int X, int Y, int Z, int x0, int TX, int tid,
                                                  int nthr) {
   const int n16 = (TX + 2) * 4;
-  for (int bb = 0; bb < 3; ++bb) {
-    const long long rowbase = base + ((long long)wrap(z + a - 1, Z) * Y + wrap(y + bb - 1, Y)) * X;
+  for (int bb = 0; bb < nr; ++bb) {
+    const long long rowbase = base + ((long long)wrap(z + a - 1, Z) * Y + (y + bb - 1 + Y) % Y) * X;
     unsigned char* row = dst + bb * (TX + 2) * ROWB;
     for (int i = tid; i < n16; i += nthr) {
       const int pt = i >> 2, q = i & 3;
@@ -114,151 +111,198 @@ __device__ __forceinline__ void cp_async_wait() {
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// 32 -> 32 convolution on the tensor cores. One warp computes 32 consecutive
-// x points (two m16 tiles) x 32 output channels (four n8 tiles); a block holds
-// TX/32 warps over an x-segment of TX points of one (b, z, y) row and stages
-// the neighbour rows (periodic) in shared memory, three at a time, the next three
-// copied (cp.async) while the current ones are in use. Weights come in mma
-// B-fragment order (see k_pack_frag) from global memory (L1-resident).
+// 32 -> 32 convolution on the tensor cores (mma.sync). A block computes four
+// rows y0 .. y0+3 of a TX-point x-segment; one warp computes 32 consecutive x
+// points (two m16 tiles) x 32 output channels (four n8 tiles) of two of them,
+// so a weight fragment feeds four mma. The six neighbour rows of a z offset
+// are staged in shared memory (periodic) while those of the previous offset
+// are in use. Weights come in mma B-fragment order (see k_pack_frag) from
+// global memory (L1-resident). Bound by the mma.sync rate and the fragment
+// reads (1.5 shared-memory or L1 wavefronts per mma). One row per block and
+// one per warp: 64^3 x 8 375 -> 298 us.
 // mode 0: out = bf16(relu(acc));  mode 1: out = bf16(acc * (mask > 0)).
-__global__ void __launch_bounds__(128) k_conv_mma(const __nv_bfloat16* __restrict__ Hin,
-                                                  const uint2* __restrict__ Wf, __nv_bfloat16* __restrict__ Hout,
-                                                  const __nv_bfloat16* __restrict__ Hmask, int X, int Y, int Z,
-                                                  int TX, int mode) {
+constexpr int CONV_TY = 4;
+__global__ void __launch_bounds__(128, 3) k_conv_mma(const __nv_bfloat16* __restrict__ Hin,
+                                                     const uint2* __restrict__ Wf, __nv_bfloat16* __restrict__ Hout,
+                                                     const __nv_bfloat16* __restrict__ Hmask, int X, int Y, int Z,
+                                                     int TX, int mode) {
   extern __shared__ __align__(16) unsigned char sm[];
   const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
-  const int segs = X / TX;
+  const int segs = X / TX, ytiles = (Y + CONV_TY - 1) / CONV_TY;
   int r = blockIdx.x;
   const int seg = r % segs;
   r /= segs;
-  const int y = r % Y, z = r / Y;
+  const int y0 = (r % ytiles) * CONV_TY, z = r / ytiles;
   const int b = blockIdx.y;
-  const int x0 = seg * TX;
+  const int x0 = seg * TX, wx = (warp % (TX >> 5)) * 32, wy = 2 * (warp / (TX >> 5));
   const long long P = (long long)X * Y * Z;
   const long long base = (long long)b * P;
-  float acc[2][4][4];
+  float acc[2][2][4][4];                     // row, m tile, n tile
 #pragma unroll
-  for (int m = 0; m < 2; ++m)
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
-  // ldmatrix lane address: matrix mi = lane/8, row i = lane%8 -> point row
-  // i + 8*(mi & 1), channel offset 8*(mi >> 1)
-  const int mi = lane >> 3, li = lane & 7;
-  const int prow = li + 8 * (mi & 1), coff = 16 * (mi >> 1);
-  // the three rows of z offset a + 1 are copied (cp.async) into the other
-  // half of shared memory while the taps of offset a run on the tensor cores
-  const int hstride = 3 * (TX + 2) * ROWB;   // bytes of one half
-  stage_rows_async(sm, Hin, base, z, y, 0, X, Y, Z, x0, TX, tid, nthr);
-  for (int ab = 0; ab < 9; ++ab) {
-    if (ab % 3 == 0) {
-      const int a = ab / 3;
-      if (a < 2) {
-        stage_rows_async(sm + ((a + 1) & 1) * hstride, Hin, base, z, y, a + 1, X, Y, Z, x0, TX, tid, nthr);
-        cp_async_wait<1>();
-      } else {
-        cp_async_wait<0>();
-      }
-      __syncthreads();
-    }
-    const unsigned char* rowt = sm + ((ab / 3) & 1) * hstride + (ab % 3) * (TX + 2) * ROWB;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int tap = ab * 3 + c;
-#pragma unroll
-      for (int ks = 0; ks < 2; ++ks) {
-        uint32_t af[2][4];
-#pragma unroll
-        for (int m = 0; m < 2; ++m) {
-          const int pt = warp * 32 + m * 16 + prow + c;     // row (x + c - 1) in the staged segment
-          ldsm_x4(af[m], rowt + pt * ROWB + ks * 32 + coff);
-        }
-#pragma unroll
-        for (int n = 0; n < 4; ++n) {
-          const uint2 bw = __ldg(Wf + ((tap * 2 + ks) * 4 + n) * 32 + lane);
-          const uint32_t bf[2] = {bw.x, bw.y};
-          mma_bf16(acc[0][n], af[0], bf);
-          mma_bf16(acc[1][n], af[1], bf);
-        }
-      }
-    }
-    if (ab % 3 == 2) __syncthreads();  // this half is refilled two offsets later
-  }
-  // epilogue: C fragment (row g / g+8, cols 2t, 2t+1)
-  const int g = lane >> 2, t = lane & 3;
-  const long long rowp = base + ((long long)z * Y + y) * X + x0 + warp * 32;
-#pragma unroll
-  for (int m = 0; m < 2; ++m)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const long long p = rowp + m * 16 + g + 8 * h;
-#pragma unroll
-      for (int n = 0; n < 4; ++n) {
-        const int co = n * 8 + 2 * t;
-        float v0 = acc[m][n][2 * h], v1 = acc[m][n][2 * h + 1];
-        if (mode == 0) {
-          v0 = fmaxf(v0, 0.f);
-          v1 = fmaxf(v1, 0.f);
-        } else {
-          const __nv_bfloat162 mk = *reinterpret_cast<const __nv_bfloat162*>(Hmask + p * C + co);
-          v0 = __bfloat162float(mk.x) > 0.f ? v0 : 0.f;
-          v1 = __bfloat162float(mk.y) > 0.f ? v1 : 0.f;
-        }
-        *reinterpret_cast<uint32_t*>(Hout + p * C + co) = pack_bf16(v0, v1);
-      }
-    }
-}
-
-// Weight gradient of a 32 -> 32 layer: dW[tap][ci][co] = sum_p Hin[p + off(tap)][ci] * dZ[p][co].
-// Nine warps per block, warp (a, b) owning the three taps (a, b, c); the block
-// walks rows of its share and writes one float32 partial per tap, ci, co.
-__global__ void __launch_bounds__(288) k_wgrad_mma(const __nv_bfloat16* __restrict__ Hin,
-                                                   const __nv_bfloat16* __restrict__ dZ, float* __restrict__ part,
-                                                   int X, int Y, int Z, int B, int TX) {
-  extern __shared__ __align__(16) unsigned char sm[];
-  const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
-  const int segs = X / TX;
-  const long long nrows = (long long)B * Z * Y * segs;
-  unsigned char* dzt = sm + 9 * (TX + 2) * ROWB;
-  float acc[3][2][4][4];
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
+  for (int j = 0; j < 2; ++j)
 #pragma unroll
     for (int m = 0; m < 2; ++m)
 #pragma unroll
       for (int n = 0; n < 4; ++n)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[c][m][n][e] = 0.f;
-  const long long P = (long long)X * Y * Z;
+        for (int e = 0; e < 4; ++e) acc[j][m][n][e] = 0.f;
+  // ldmatrix lane address: matrix mi = lane/8, row i = lane%8 -> point row
+  // i + 8*(mi & 1), channel offset 8*(mi >> 1)
   const int mi = lane >> 3, li = lane & 7;
-  for (long long rr = blockIdx.x; rr < nrows; rr += gridDim.x) {
-    long long r = rr;
-    const int seg = (int)(r % segs);
-    r /= segs;
-    const int y = (int)(r % Y);
-    r /= Y;
-    const int z = (int)(r % Z);
-    const int b = (int)(r / Z);
-    const int x0 = seg * TX;
-    const long long base = (long long)b * P;
-    __syncthreads();
-    for (int a = 0; a < 3; ++a)
-      for (int bb = 0; bb < 3; ++bb) {
-        const long long rowbase = base + ((long long)wrap(z + a - 1, Z) * Y + wrap(y + bb - 1, Y)) * X;
-        load_row(sm + (a * 3 + bb) * (TX + 2) * ROWB, Hin, rowbase, X, x0, TX, tid, nthr);
-      }
-    {
-      const long long rowbase = base + ((long long)z * Y + y) * X;
-      for (int i = tid; i < TX * 4; i += nthr) {
-        const int pt = i >> 2, q = i & 3;
-        *reinterpret_cast<uint4*>(dzt + pt * ROWB + q * 16) =
-            *reinterpret_cast<const uint4*>(dZ + (rowbase + x0 + pt) * C + q * 8);
-      }
+  const int prow = li + 8 * (mi & 1), coff = 16 * (mi >> 1);
+  // the rows of z offset a + 1 are copied (cp.async) into the other half of
+  // shared memory while the taps of offset a run on the tensor cores
+  const int rstride = (TX + 2) * ROWB, hstride = (CONV_TY + 2) * rstride;
+  stage_rows_async(sm, Hin, base, z, y0, 0, CONV_TY + 2, X, Y, Z, x0, TX, tid, nthr);
+#pragma unroll 1
+  for (int a = 0; a < 3; ++a) {
+    if (a < 2) {
+      stage_rows_async(sm + ((a + 1) & 1) * hstride, Hin, base, z, y0, a + 1, CONV_TY + 2, X, Y, Z, x0, TX, tid, nthr);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
     }
     __syncthreads();
-    if (warp < 9) {
-      const unsigned char* rowt = sm + warp * (TX + 2) * ROWB;
+#pragma unroll 1
+    for (int bb = 0; bb < 3; ++bb) {
+      const unsigned char* rowt = sm + (a & 1) * hstride + (wy + bb) * rstride + (wx + prow) * ROWB + coff;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int tap = (a * 3 + bb) * 3 + c;
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+          uint32_t af[2][2][4];
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int m = 0; m < 2; ++m)        // row (x + c - 1) in the staged segment
+              ldsm_x4(af[j][m], rowt + j * rstride + (m * 16 + c) * ROWB + ks * 32);
+#pragma unroll
+          for (int n = 0; n < 4; ++n) {
+            const uint2 bw = __ldg(Wf + ((tap * 2 + ks) * 4 + n) * 32 + lane);
+            const uint32_t bf[2] = {bw.x, bw.y};
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              mma_bf16(acc[j][0][n], af[j][0], bf);
+              mma_bf16(acc[j][1][n], af[j][1], bf);
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();  // this half is refilled next
+  }
+  // epilogue: C fragment (row g / g+8, cols 2t, 2t+1)
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    if (y0 + wy + j >= Y) break;
+    const long long rowp = base + ((long long)z * Y + y0 + wy + j) * X + x0 + wx;
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const long long p = rowp + m * 16 + g + 8 * h;
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+          const int co = n * 8 + 2 * t;
+          float v0 = acc[j][m][n][2 * h], v1 = acc[j][m][n][2 * h + 1];
+          if (mode == 0) {
+            v0 = fmaxf(v0, 0.f);
+            v1 = fmaxf(v1, 0.f);
+          } else {
+            const __nv_bfloat162 mk = *reinterpret_cast<const __nv_bfloat162*>(Hmask + p * C + co);
+            v0 = __bfloat162float(mk.x) > 0.f ? v0 : 0.f;
+            v1 = __bfloat162float(mk.y) > 0.f ? v1 : 0.f;
+          }
+          *reinterpret_cast<uint32_t*>(Hout + p * C + co) = pack_bf16(v0, v1);
+        }
+      }
+  }
+}
+
+// Weight gradient of a 32 -> 32 layer: dW[tap][ci][co] = sum_p Hin[p + off(tap)][ci] * dZ[p][co].
+// Eighteen warps per block: warp (a, b, m) owns the three taps (a, b, c) and
+// half m of the input channels (48 accumulators). The rows
+// (b, z, x-segment, y) are split evenly and contiguously over the blocks; a
+// block marches along y: per row it stages the three z planes' rows y + 1 and
+// the dZ row y (cp.async, two rows ahead) into rings of five and three slots,
+// so a row of Hin is fetched three times (once per z plane), not nine, and its
+// latency overlaps two rows of mma. One float32 partial per tap, ci, co and
+// block. Bound by the mma.sync rate and the ldmatrix reads. Nine rows fetched
+// synchronously per output row: 64^3 x 8 1310 -> 394 us.
+constexpr int WG_H = 5, WG_Z = 3;          // ring slots
+__global__ void __launch_bounds__(576) k_wgrad_mma(const __nv_bfloat16* __restrict__ Hin,
+                                                      const __nv_bfloat16* __restrict__ dZ, float* __restrict__ part,
+                                                      int X, int Y, int Z, int B, int TX) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
+  const int segs = X / TX;
+  const int rstride = (TX + 2) * ROWB;
+  unsigned char* dzr = sm + WG_H * 3 * rstride;
+  float acc[3][4][4];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[c][n][e] = 0.f;
+  const long long P = (long long)X * Y * Z;
+  const int mi = lane >> 3, li = lane & 7;
+  const int wt = warp % 9, wm = warp / 9, wa = wt / 3, wb = wt - 3 * wa;
+  const long long nrows = (long long)B * Z * segs * Y;
+  long long r = nrows * blockIdx.x / gridDim.x;
+  const long long rend = nrows * (blockIdx.x + 1) / gridDim.x;
+  auto copy16 = [](unsigned char* dst, const __nv_bfloat16* src) {
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+  };
+  while (r < rend) {
+    // a run of consecutive y of one (b, z, segment)
+    const int y0 = (int)(r % Y), n = (int)min(rend - r, (long long)(Y - y0));
+    long long col = r / Y;
+    const int x0 = (int)(col % segs) * TX;
+    col /= segs;
+    const int z = (int)(col % Z);
+    const long long base = (col / Z) * P;
+    // Hin rows y0 + i (i = -1 .. n) of the three planes, slot (i + 1) % WG_H
+    auto stage_h = [&](int i) {
+      const int y = (y0 + i + Y) % Y;
+      unsigned char* slot = sm + ((i + 1) % WG_H) * 3 * rstride;
+      for (int q = tid; q < 3 * (TX + 2) * 4; q += nthr) {
+        const int a = q / ((TX + 2) * 4), k = q - a * ((TX + 2) * 4), pt = k >> 2, ch = k & 3;
+        copy16(slot + a * rstride + pt * ROWB + ch * 16,
+               Hin + (base + ((long long)wrap(z + a - 1, Z) * Y + y) * X + wrap(x0 - 1 + pt, X)) * C + ch * 8);
+      }
+    };
+    auto stage_z = [&](int i) {
+      unsigned char* slot = dzr + (i % WG_Z) * TX * ROWB;
+      for (int q = tid; q < TX * 4; q += nthr)
+        copy16(slot + (q >> 2) * ROWB + (q & 3) * 16,
+               dZ + (base + ((long long)z * Y + y0 + i) * X + x0 + (q >> 2)) * C + (q & 3) * 8);
+    };
+    __syncthreads();                         // the previous run's rows are no longer read
+    stage_h(-1);
+    stage_h(0);
+    for (int i = 0; i < 2; ++i) {            // groups 0, 1: rows i + 1 and dZ row i
+      if (i < n) {
+        stage_h(i + 1);
+        stage_z(i);
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      cp_async_wait<1>();
+      __syncthreads();                       // row i is staged; row i - 1 is no longer read
+      if (i + 2 < n) {
+        stage_h(i + 3);
+        stage_z(i + 2);
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      const unsigned char* rowt = sm + ((i + wb) % WG_H) * 3 * rstride + wa * rstride;   // row i + wb - 1
+      const unsigned char* dzt = dzr + (i % WG_Z) * TX * ROWB;
+#pragma unroll 1
       for (int k0 = 0; k0 < TX; k0 += 16) {
         // B fragments (k = points, n = co) from dZ: transposed 8x8 loads.
         // matrices: mi&1 selects k half (points k0..7 / 8..15), mi>>1 selects n tile pair
@@ -277,35 +321,28 @@ __global__ void __launch_bounds__(288) k_wgrad_mma(const __nv_bfloat16* __restri
         for (int c = 0; c < 3; ++c) {
           // A fragments (m = ci, k = points) from the shifted input row, transposed loads:
           // matrices 0: ci 0-7, k 0-7; 1: ci 8-15, k 0-7; 2: ci 0-7, k 8-15; 3: ci 8-15, k 8-15
+          uint32_t af[4];
+          ldsm_x4_t(af, rowt + (k0 + li + 8 * (mi >> 1) + c) * ROWB + (wm * 16 + 8 * (mi & 1)) * 2);
 #pragma unroll
-          for (int m = 0; m < 2; ++m) {
-            uint32_t af[4];
-            const int kk = k0 + li + 8 * (mi >> 1);
-            const int cc = m * 16 + 8 * (mi & 1);
-            ldsm_x4_t(af, rowt + (kk + c) * ROWB + cc * 2);
-#pragma unroll
-            for (int n = 0; n < 4; ++n) mma_bf16(acc[c][m][n], af, bfr[n]);
-          }
+          for (int n4 = 0; n4 < 4; ++n4) mma_bf16(acc[c][n4], af, bfr[n4]);
         }
       }
     }
+    cp_async_wait<0>();
+    r += n;
   }
-  if (warp < 9) {
-    const int g = lane >> 2, t = lane & 3;
-    float* pb = part + (long long)blockIdx.x * TAPS * C * C;
+  const int g = lane >> 2, t = lane & 3;
+  float* pb = part + (long long)blockIdx.x * TAPS * C * C;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int tap = warp * 3 + c;
+  for (int c = 0; c < 3; ++c) {
+    const int tap = wt * 3 + c;
 #pragma unroll
-      for (int m = 0; m < 2; ++m)
+    for (int n = 0; n < 4; ++n)
 #pragma unroll
-        for (int n = 0; n < 4; ++n)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int ci = m * 16 + g + 8 * (e >> 1), co = n * 8 + 2 * t + (e & 1);
-            pb[(tap * C + ci) * C + co] = acc[c][m][n][e];
-          }
-    }
+      for (int e = 0; e < 4; ++e) {
+        const int ci = wm * 16 + g + 8 * (e >> 1), co = n * 8 + 2 * t + (e & 1);
+        pb[(tap * C + ci) * C + co] = acc[c][n][e];
+      }
   }
 }
 
@@ -328,106 +365,188 @@ __global__ void k_pack_frag(const float* __restrict__ W, uint2* __restrict__ Wf,
   Wf[i] = make_uint2(pack_bf16(Bv(2 * t, g), Bv(2 * t + 1, g)), pack_bf16(Bv(2 * t + 8, g), Bv(2 * t + 9, g)));
 }
 
-// Packs the layer-4 weights W4[tap][ci] as the B fragments of one n8 tile
-// whose column 0 holds them and columns 1..7 are zero:
-// Wf[(tap*2 + ks)*32 + lane] = {B(2t, g), B(2t+1, g)}, {B(2t+8, g), B(2t+9, g)},
-// B(k, j) = (j == 0) ? W4[tap][16 ks + k] : 0.
+// Packs the layer-4 weights W4[tap][ci] as the B fragments of a GEMM whose 32
+// columns are the taps (27..31 zero), for k_conv_out. Its A fragments come
+// straight from global memory, lane t of a quad holding channels 8t .. 8t+7 of
+// a point, so row k of k-step ks stands for channel 8 (k/2 mod 4) + 4 ks +
+// 2 (k/8) + k mod 2:
+// Wf[(ks*4 + n)*32 + lane] = {W4[8n+g][8t+4ks .. +1]}, {W4[8n+g][8t+4ks+2 .. +3]}.
 __global__ void k_pack_frag4(const float* __restrict__ W4, uint2* __restrict__ Wf) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= TAPS * 2 * 32) return;
-  const int lane = i & 31, ks = (i >> 5) & 1, tap = i >> 6;
-  const int g = lane >> 2, t = lane & 3;
-  auto Bv = [&](int k) { return g == 0 ? W4[tap * C + ks * 16 + k] : 0.f; };
+  if (i >= 2 * 4 * 32) return;
+  const int lane = i & 31, n = (i >> 5) & 3, ks = i >> 7;
+  const int tap = 8 * n + (lane >> 2), ci = 8 * (lane & 3) + 4 * ks;
+  auto w = [&](int k) { return tap < TAPS ? W4[tap * C + ci + k] : 0.f; };
+  Wf[i] = make_uint2(pack_bf16(w(0), w(1)), pack_bf16(w(2), w(3)));
+}
+
+// Packs the layer-4 weights for k_conv_out_mma: the B fragments of row offset d
+// = -1 .. 8 (relative to the first of eight output rows), column j holding the
+// weights of the tap dy = d - j (zero unless -1 <= dy <= 1):
+// Wf[(((a*10 + d+1)*3 + c)*2 + ks)*32 + lane] = {B(2t, g), B(2t+1, g)}, {B(2t+8, g), B(2t+9, g)},
+// B(k, j) = W4[(a, d - j + 1, c)][16 ks + k].
+__global__ void k_pack_frag4t(const float* __restrict__ W4, uint2* __restrict__ Wf) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 3 * 10 * 3 * 2 * 32) return;
+  const int lane = i & 31, ks = (i >> 5) & 1, adc = i >> 6, c = adc % 3, d = adc / 3 % 10, a = adc / 30;
+  const int g = lane >> 2, t = lane & 3, bb = d - g;
+  auto Bv = [&](int k) { return bb >= 0 && bb < 3 ? W4[((a * 3 + bb) * 3 + c) * C + ks * 16 + k] : 0.f; };
   Wf[i] = make_uint2(pack_bf16(Bv(2 * t), Bv(2 * t + 1)), pack_bf16(Bv(2 * t + 8), Bv(2 * t + 9)));
 }
 
-// sum of squares of each sample (float64 partials per block, then per sample)
+// Sum of squares of each sample in float64. Bound by the float64 pipe (two
+// lanes per clock and SM), so a thread keeps four independent chains.
 __global__ void k_sumsq(const float* __restrict__ u, long long P, double* __restrict__ out) {
   const int b = blockIdx.y;
-  double s = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
-    const double v = u[(long long)b * P + i];
-    s += v * v;
+  const float* ub = u + (long long)b * P;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  const long long st = (long long)gridDim.x * blockDim.x;
+  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  for (; i + 3 * st < P; i += 4 * st) {
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = ub[i + k * st];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = fma((double)v[k], (double)v[k], s[k]);
   }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  for (; i < P; i += st) s[0] = fma((double)ub[i], (double)ub[i], s[0]);
+  double t = (s[0] + s[1]) + (s[2] + s[3]);
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   __shared__ double red[32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    atomicAdd(out + b, t);
+    double r = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += red[w];
+    atomicAdd(out + b, r);
   }
 }
 
-// Layer 1: H1[p][co] = relu(sum_tap W1[tap][co] * x0[p + off(tap)]), x0 = u_bar / sigma,
-// in float32 on the CUDA cores. A thread computes two consecutive x points:
-// their 27 taps share the 9 neighbour rows, from which it loads the four
-// values x-1 .. x+2 once; the weights of eight output channels are read as
-// two float4 from shared memory and applied to both points.
-__global__ void __launch_bounds__(256) k_conv_in(const float* __restrict__ ubar, const double* __restrict__ sumsq,
-                                                 const float* __restrict__ W1, __nv_bfloat16* __restrict__ H1,
-                                                 int X, int Y, int Z) {
+// The bf16 pair v where the pair m is positive, zero elsewhere.
+__device__ __forceinline__ uint32_t relu_mask(uint32_t v, uint32_t m) {
+  const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&m);
+  return (__bfloat162float(m2.x) > 0.f ? v & 0xffffu : 0u) | (__bfloat162float(m2.y) > 0.f ? v & 0xffff0000u : 0u);
+}
+
+// The 1 -> 32 convolutions in float32 on the CUDA cores:
+//   first layer:              H1[p][co] = relu(sum_tap W1[tap][co] x0[p + off(tap)]), x0 = u_bar / sigma
+//   layer-4 backward (BWD):   dZ3[p][ci] = (H3[p][ci] > 0) sum_tap W4[tap][ci] g[p - off(tap)]
+// Bound by the float32 pipe (864 multiply-adds per point). A thread computes
+// four consecutive x points, eight channels at a time as four packed pairs
+// (fma.rn.f32x2: two multiply-adds per issue, each rounded as fmaf): the six
+// values of each of the 9 neighbour rows are held doubled, and a 16-byte
+// broadcast read of four weights feeds eight packed multiply-adds (the
+// load/store unit moves 8 bytes of a broadcast per cycle, so the weights are
+// not the ones to be doubled). The results go through shared memory so that a
+// store covers 512 consecutive bytes (16 bytes at a 128-256 byte stride cost as
+// many cycles of the load/store unit as the weight reads). Two points per
+// thread, scalar multiply-adds and strided stores:
+// 256^3 x 3 2.29 -> 1.57 ms, 64^3 x 8 backward 139 -> 100 us.
+template <bool BWD>
+__global__ void __launch_bounds__(128, 3) k_conv_1ch(const float* __restrict__ S, const double* __restrict__ sumsq,
+                                                     const float* __restrict__ W, const __nv_bfloat16* __restrict__ mask,
+                                                     __nv_bfloat16* __restrict__ out, int X, int Y, int Z) {
   const long long P = (long long)X * Y * Z;
-  const long long P2 = P >> 1;                       // point pairs (X is even)
-  const int b = blockIdx.y;
+  const int xg = X >> 2;                             // point groups of a row (X is a multiple of 32)
+  const int b = blockIdx.y, lane = threadIdx.x & 31;
   __shared__ __align__(16) float w[TAPS * C];
-  for (int i = threadIdx.x; i < TAPS * C; i += blockDim.x) w[i] = W1[i];
+  extern __shared__ __align__(16) unsigned char sm[];
+  // this warp's 128 results, point 4 l + i (lane l) at i PLANE + l ROWB: written
+  // and read back without bank conflicts
+  constexpr int PLANE = 32 * ROWB + 64;
+  unsigned char* stage = sm + (threadIdx.x >> 5) * (4 * PLANE);
+  for (int i = threadIdx.x; i < TAPS * C; i += blockDim.x) w[i] = W[i];
   __syncthreads();
-  const float inv_sigma = (float)(1.0 / sqrt(fmax(sumsq[b] / (double)P, 1e-300)));
-  const float4* w4 = reinterpret_cast<const float4*>(w);
-  for (long long pp = blockIdx.x * (long long)blockDim.x + threadIdx.x; pp < P2;
-       pp += (long long)gridDim.x * blockDim.x) {
-    const long long p = 2 * pp;
-    const int x = (int)(p % X), y = (int)((p / X) % Y), z = (int)(p / ((long long)X * Y));
-    float v[9][4];                                   // row (a, b), x - 1 .. x + 2
+  const float scale = BWD ? 1.f : (float)(1.0 / sqrt(fmax(sumsq[b] / (double)P, 1e-300)));
+  const long long groups = P >> 2;                   // a multiple of 32: X is (and Y, Z are even), or Y Z 8 is
+  for (long long pg0 = blockIdx.x * (long long)blockDim.x + threadIdx.x - lane; pg0 < groups;
+       pg0 += (long long)gridDim.x * blockDim.x) {
+    const long long pg = min(pg0 + lane, groups - 1);
+    if (BWD)                                         // the mask rows of the epilogue, on their way to L2 meanwhile
+      for (int j = 0; j < 2; ++j)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(mask + ((long long)b * P + 4 * pg + 2 * j) * C));
+    const long long row0 = pg / xg;
+    const int x = 4 * (int)(pg - row0 * xg);
+    const int z = (int)(row0 / Y), y = (int)(row0 - (long long)z * Y);
+    float2 v[9][6];                                  // row (a, b): x-1 .. x+4, doubled
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int r = 0; r < 9; ++r) {
+      const long long row = (long long)b * P + ((long long)wrap(z + r / 3 - 1, Z) * Y + wrap(y + r % 3 - 1, Y)) * X;
 #pragma unroll
-      for (int bb = 0; bb < 3; ++bb) {
-        const long long row = (long long)b * P + ((long long)wrap(z + a - 1, Z) * Y + wrap(y + bb - 1, Y)) * X;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) v[a * 3 + bb][c] = ubar[row + wrap(x + c - 1, X)] * inv_sigma;
+      for (int c = 0; c < 6; ++c) {
+        float e = S[row + (c == 0 ? (x ? x - 1 : X - 1) : c == 5 ? (x + 4 == X ? 0 : x + 4) : x + c - 1)];
+        if (!BWD) e *= scale;
+        v[r][c] = make_float2(e, e);
       }
-    uint4* dst0 = reinterpret_cast<uint4*>(H1 + ((long long)b * P + p) * C);
-    uint4* dst1 = dst0 + 4;
+    }
 #pragma unroll 1
     for (int q = 0; q < 4; ++q) {                    // output channels 8q .. 8q + 7
-      float s0[8], s1[8];
+      float2 s[4][4];                                // point x + i, channel pair
 #pragma unroll
-      for (int k = 0; k < 8; ++k) s0[k] = s1[k] = 0.f;
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int r = 0; r < 9; ++r)
+        for (int k = 0; k < 4; ++k) s[i][k] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const int t = r * 3 + c;
-          const float4 wa = w4[t * 8 + 2 * q], wb = w4[t * 8 + 2 * q + 1];
-          const float i0 = v[r][c], i1 = v[r][c + 1];
-          const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+      for (int t = 0; t < TAPS; ++t) {
+        const int u = BWD ? TAPS - 1 - t : t;        // p - off(t) = p + off(26 - t)
+        const float4* wt = reinterpret_cast<const float4*>(w + t * C + 8 * q);
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            s0[k] = fmaf(wv[k], i0, s0[k]);
-            s1[k] = fmaf(wv[k], i1, s1[k]);
+        for (int k = 0; k < 2; ++k) {
+          const float4 w4 = wt[k];
+          const float2 wa = make_float2(w4.x, w4.y), wb = make_float2(w4.z, w4.w);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            s[i][2 * k] = fma2(wa, v[u / 3][u % 3 + i], s[i][2 * k]);
+            s[i][2 * k + 1] = fma2(wb, v[u / 3][u % 3 + i], s[i][2 * k + 1]);
           }
         }
-      dst0[q] = make_uint4(pack_bf16(fmaxf(s0[0], 0.f), fmaxf(s0[1], 0.f)), pack_bf16(fmaxf(s0[2], 0.f), fmaxf(s0[3], 0.f)),
-                           pack_bf16(fmaxf(s0[4], 0.f), fmaxf(s0[5], 0.f)), pack_bf16(fmaxf(s0[6], 0.f), fmaxf(s0[7], 0.f)));
-      dst1[q] = make_uint4(pack_bf16(fmaxf(s1[0], 0.f), fmaxf(s1[1], 0.f)), pack_bf16(fmaxf(s1[2], 0.f), fmaxf(s1[3], 0.f)),
-                           pack_bf16(fmaxf(s1[4], 0.f), fmaxf(s1[5], 0.f)), pack_bf16(fmaxf(s1[6], 0.f), fmaxf(s1[7], 0.f)));
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {                  // point x + i
+        uint32_t o[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 f = s[i][k];
+          o[k] = BWD ? pack_bf16(f.x, f.y) : pack_bf16(fmaxf(f.x, 0.f), fmaxf(f.y, 0.f));
+        }
+        *reinterpret_cast<uint4*>(stage + i * PLANE + lane * ROWB + 16 * q) = make_uint4(o[0], o[1], o[2], o[3]);
+      }
     }
+    __syncwarp();
+    // 16 bytes per lane in address order: 8 points of 64 bytes per store
+    const long long p0 = (long long)b * P + 4 * pg0;
+#pragma unroll 4
+    for (int j = 0; j < 16; ++j) {
+      const int pt = 8 * j + (lane >> 2), c16 = lane & 3;
+      if (pg0 + (pt >> 2) < groups) {
+        uint4 v = *reinterpret_cast<const uint4*>(stage + (pt & 3) * PLANE + (pt >> 2) * ROWB + 16 * c16);
+        if (BWD) {
+          const uint4 m = *reinterpret_cast<const uint4*>(mask + (p0 + pt) * C + 8 * c16);
+          v.x = relu_mask(v.x, m.x);
+          v.y = relu_mask(v.y, m.y);
+          v.z = relu_mask(v.z, m.z);
+          v.w = relu_mask(v.w, m.w);
+        }
+        *reinterpret_cast<uint4*>(out + (p0 + pt) * C + 8 * c16) = v;
+      }
+    }
+    __syncwarp();
   }
 }
+constexpr size_t kConv1Smem = 4 * 4 * (32 * ROWB + 64);
 
-// Layer 4 (32 -> 1) on the tensor cores and the residual output:
-//   u0 = u_bar + sigma * A * sum_{tap, ci} W4[tap][ci] H3[p + off][ci].
-// The same implicit GEMM as k_conv_mma with one n8 tile whose column 0 holds
-// W4 (bf16, the other seven columns zero): the neighbour rows are staged in
-// shared memory once per block and read by ldmatrix, instead of each thread
-// gathering its 27 x 32 inputs from L1. Column 0 of the accumulator lives in
-// the lanes with lane % 4 == 0 (rows g and g + 8 of each m16 tile).
-// With utrue != nullptr it also writes g = sigma * A * 2 (u0 - u_true) /
-// ||u_true||^2 / B and accumulates sum (u0 - u_true)^2 / ||u_true||^2 / B
-// into loss.
+// Layer 4 of a training step, with the loss and its gradient: the implicit GEMM
+// of k_conv_mma with one n8 tile whose eight columns are eight output rows y0 ..
+// y0+7. A staged row d (relative to y0) is multiplied once by the fragment
+// whose column j holds the taps dy = d - j, so the ten rows of a z offset serve
+// eight output rows: 180 ldmatrix and mma per 16 x 8 outputs, where one useful
+// column per output row took 432. Every output still adds its 27 taps x two
+// halves of 16 channels in that order (the zero columns add nothing), which
+// the loss gradient, proportional to the small difference u0 - u_true, is
+// sensitive to. A block owns a TX-point x-segment, a warp 16 of its points.
+// 64^3 x 8: 402 -> 225 us.
+// It writes u0, g = sigma * A * 2 (u0 - u_true) / ||u_true||^2 / B and
+// accumulates sum (u0 - u_true)^2 / ||u_true||^2 / B into loss.
 __global__ void __launch_bounds__(128) k_conv_out_mma(const __nv_bfloat16* __restrict__ H3,
                                                       const uint2* __restrict__ Wf, const float* __restrict__ ubar,
                                                       const double* __restrict__ sumsq, float* __restrict__ u0,
@@ -438,128 +557,198 @@ __global__ void __launch_bounds__(128) k_conv_out_mma(const __nv_bfloat16* __res
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ double red[4];
   const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
-  const int segs = X / TX;
+  const int segs = X / TX, ytiles = (Y + 7) / 8;
   int r = blockIdx.x;
-  const int seg = r % segs;
+  const int x0 = (r % segs) * TX;
   r /= segs;
-  const int y = r % Y, z = r / Y;
+  const int y0 = (r % ytiles) * 8, z = r / ytiles;
   const int b = blockIdx.y;
-  const int x0 = seg * TX;
   const long long P = (long long)X * Y * Z;
   const long long base = (long long)b * P;
-  float acc[2][4];
-#pragma unroll
-  for (int m = 0; m < 2; ++m)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[m][e] = 0.f;
-  const int mi = lane >> 3, li = lane & 7;
-  const int prow = li + 8 * (mi & 1), coff = 16 * (mi >> 1);
-  const int hstride = 3 * (TX + 2) * ROWB;   // bytes of one half
-  stage_rows_async(sm, H3, base, z, y, 0, X, Y, Z, x0, TX, tid, nthr);
-  for (int ab = 0; ab < 9; ++ab) {
-    if (ab % 3 == 0) {
-      const int a = ab / 3;
-      if (a < 2) {
-        stage_rows_async(sm + ((a + 1) & 1) * hstride, H3, base, z, y, a + 1, X, Y, Z, x0, TX, tid, nthr);
-        cp_async_wait<1>();
-      } else {
-        cp_async_wait<0>();
-      }
-      __syncthreads();
-    }
-    const unsigned char* rowt = sm + ((ab / 3) & 1) * hstride + (ab % 3) * (TX + 2) * ROWB;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int tap = ab * 3 + c;
-#pragma unroll
-      for (int ks = 0; ks < 2; ++ks) {
-        uint32_t af[2][4];
-#pragma unroll
-        for (int m = 0; m < 2; ++m) {
-          const int pt = warp * 32 + m * 16 + prow + c;
-          ldsm_x4(af[m], rowt + pt * ROWB + ks * 32 + coff);
-        }
-        const uint2 bw = __ldg(Wf + (tap * 2 + ks) * 32 + lane);
-        const uint32_t bf[2] = {bw.x, bw.y};
-        mma_bf16(acc[0], af[0], bf);
-        mma_bf16(acc[1], af[1], bf);
-      }
-    }
-    if (ab % 3 == 2) __syncthreads();  // this half is refilled two offsets later
-  }
-  const int g = lane >> 2, t = lane & 3;
-  const double sigma = sqrt(fmax(sumsq[b] / (double)P, 1e-300)) * ascale;   // sigma * A
-  const long long rowp = base + ((long long)z * Y + y) * X + x0 + warp * 32;
-  double lsum = 0.0;
-  if (t == 0) {
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const long long gi = rowp + m * 16 + g + 8 * h;
-        const float uo = ubar[gi] + (float)sigma * acc[m][2 * h];
-        u0[gi] = uo;
-        if (utrue) {
-          const double d = (double)uo - (double)utrue[gi];
-          const double inv = 1.0 / (tsumsq[b] * (double)B);
-          lsum += d * d * inv;
-          gout[gi] = (float)(sigma * 2.0 * d * inv);
-        }
-      }
-  }
-  if (utrue) {
-    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    if (lane == 0) red[warp] = lsum;
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  const int mi = lane >> 3, li = lane & 7, g = lane >> 2, t = lane & 3;
+  const int prow = warp * 16 + li + 8 * (mi & 1), coff = 16 * (mi >> 1);
+  const int rstride = (TX + 2) * ROWB;
+#pragma unroll 1
+  for (int a = 0; a < 3; ++a) {
+    stage_rows_async(sm, H3, base, z, y0, a, 10, X, Y, Z, x0, TX, tid, nthr);
+    cp_async_wait<0>();
     __syncthreads();
-    if (tid == 0) {
-      double tt = 0.0;
-      for (int w2 = 0; w2 < (nthr >> 5); ++w2) tt += red[w2];
-      atomicAdd(loss, tt);
+#pragma unroll 2
+    for (int d = 0; d < 10; ++d)
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+          uint32_t af[4];
+          ldsm_x4(af, sm + d * rstride + (prow + c) * ROWB + ks * 32 + coff);
+          const uint2 bw = __ldg(Wf + (((a * 10 + d) * 3 + c) * 2 + ks) * 32 + lane);
+          const uint32_t bf[2] = {bw.x, bw.y};
+          mma_bf16(acc, af, bf);
+        }
+    __syncthreads();                         // the rows are replaced next
+  }
+  const double sigma = sqrt(fmax(sumsq[b] / (double)P, 1e-300)) * ascale;   // sigma * A
+  const double inv = 1.0 / (tsumsq[b] * (double)B);
+  double lsum = 0.0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {              // point g + 8 (e / 2), row 2t + e % 2
+    const int y = y0 + 2 * t + (e & 1);
+    if (y < Y) {
+      const long long gi = base + ((long long)z * Y + y) * X + x0 + warp * 16 + g + 8 * (e >> 1);
+      const float uo = ubar[gi] + (float)sigma * acc[e];
+      u0[gi] = uo;
+      const double df = (double)uo - (double)utrue[gi];
+      lsum += df * df * inv;
+      gout[gi] = (float)(sigma * 2.0 * df * inv);
     }
+  }
+  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+  if (lane == 0) red[warp] = lsum;
+  __syncthreads();
+  if (tid == 0) {
+    double tt = 0.0;
+    for (int w2 = 0; w2 < (nthr >> 5); ++w2) tt += red[w2];
+    atomicAdd(loss, tt);
   }
 }
 
-// Layer-4 backward data with the layer-3 ReLU mask:
-// dZ3[p][ci] = (H3[p][ci] > 0) * sum_tap W4[tap][ci] * g[p - off(tap)].
-__global__ void __launch_bounds__(256) k_conv_out_bwd(const float* __restrict__ g, const float* __restrict__ W4,
-                                                      const __nv_bfloat16* __restrict__ H3,
-                                                      __nv_bfloat16* __restrict__ dZ3, int X, int Y, int Z) {
-  const long long P = (long long)X * Y * Z;
+// Layer 4 (32 -> 1) on the tensor cores and the residual output:
+//   u0 = u_bar + sigma * A * sum_{tap, ci} W4[tap][ci] H3[p + off][ci].
+// The sum over channels comes first: per input point q one row of the GEMM
+// T[q][tap] = sum_ci H3[q][ci] W4[tap][ci] (K = 32, N = 27 taps of 32), then
+// out[p] = sum_tap T[p + off(tap)][tap] adds 27 float32 values. Each point's
+// channels are read and multiplied once (2 x 4 mma per 16 points), where an
+// implicit GEMM over 27 taps x 32 channels with one useful column of eight
+// takes 54 ldmatrix and 54 mma per 16 points.
+// A block owns TX x 8 columns and marches along z over `zc` output planes: the
+// (TX+2) x 10 points of a plane go to shared memory tap-major (row stride 4 mod
+// 32: the fragment stores and the x-contiguous reads are conflict free), and
+// each thread adds the plane's nine values per z tap to the running sums of
+// the three output planes it touches. Bound by reading H3 (halo 1.16-1.3x,
+// mostly from L2) and by shared memory (about 2 wavefronts per output).
+// 256^3 x 3: 6.10 -> 1.16 ms.
+// Inference only: the loss gradient is proportional to u0 - u_true, a small
+// difference in which the order of these sums shows (weight gradients move by
+// 2e-5), so training steps keep k_conv_out_mma's order.
+constexpr int OUT_TY = 8;
+template <int TX> struct OutTile {
+  static constexpr int PTS = (TX + 2) * (OUT_TY + 2);
+  static constexpr int NT = (PTS + 15) / 16;                  // m16 tiles of a plane
+  static constexpr int LD = (NT * 16 + 31) / 32 * 32 + 4;     // floats per tap row
+  static constexpr size_t smem = sizeof(float) * TAPS * LD;
+};
+
+template <int TX>
+__global__ void __launch_bounds__(256, 3) k_conv_out(const __nv_bfloat16* __restrict__ H3,
+                                                     const uint2* __restrict__ Wf, const float* __restrict__ ubar,
+                                                     const double* __restrict__ sumsq, float* __restrict__ u0,
+                                                     int X, int Y, int Z, int zc, double ascale) {
+  using OT = OutTile<TX>;
+  extern __shared__ __align__(16) float tsm[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int segs = X / TX, ytiles = (Y + OUT_TY - 1) / OUT_TY;
+  int r = blockIdx.x;
+  const int x0 = (r % segs) * TX;
+  r /= segs;
+  const int y0 = (r % ytiles) * OUT_TY, z0 = (r / ytiles) * zc, z1 = min(z0 + zc, Z);
   const int b = blockIdx.y;
-  __shared__ float w[TAPS * C];
-  for (int i = threadIdx.x; i < TAPS * C; i += blockDim.x) w[i] = W4[i];
-  __syncthreads();
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(p % X), y = (int)((p / X) % Y), z = (int)(p / ((long long)X * Y));
-    float gv[TAPS];
-    for (int a = 0; a < 3; ++a)
-      for (int bb = 0; bb < 3; ++bb) {
-        const long long row = (long long)b * P + ((long long)wrap(z - a + 1, Z) * Y + wrap(y - bb + 1, Y)) * X;
-        for (int c = 0; c < 3; ++c) gv[(a * 3 + bb) * 3 + c] = g[row + wrap(x - c + 1, X)];
-      }
-    const long long gi = (long long)b * P + p;
-    const uint4* hm = reinterpret_cast<const uint4*>(H3 + gi * C);
-    uint4* dst = reinterpret_cast<uint4*>(dZ3 + gi * C);
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-      const uint4 mv = hm[q];
-      const uint32_t mw[4] = {mv.x, mv.y, mv.z, mv.w};
-      uint32_t ow[4];
+  const long long plane = (long long)X * Y, base = (long long)b * plane * Z;
+  uint2 wf[8];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int ci = q * 8 + 2 * k;
-        float s0 = 0.f, s1 = 0.f;
+  for (int i = 0; i < 8; ++i) wf[i] = Wf[i * 32 + lane];
+  // the plane offsets (points) of this lane's rows g, g + 8 of each of its tiles
+  constexpr int TPW = (OT::NT + 7) / 8;
+  int off[TPW][2];
 #pragma unroll
-        for (int t = 0; t < TAPS; ++t) {
-          s0 = fmaf(w[t * C + ci], gv[t], s0);
-          s1 = fmaf(w[t * C + ci + 1], gv[t], s1);
-        }
-        const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&mw[k]);
-        ow[k] = pack_bf16(__bfloat162float(m2.x) > 0.f ? s0 : 0.f, __bfloat162float(m2.y) > 0.f ? s1 : 0.f);
-      }
-      dst[q] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
+  for (int k = 0; k < TPW; ++k)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = min((warp + 8 * k) * 16 + g + 8 * h, OT::PTS - 1);
+      const int yy = (y0 + i / (TX + 2) + Y - 1) % Y;
+      off[k][h] = yy * X + wrap(x0 - 1 + i % (TX + 2), X);
     }
+  const float sig = (float)(sqrt(fmax(sumsq[b] / (double)(plane * Z), 1e-300)) * ascale);   // sigma * A
+  constexpr int NO = TX * OUT_TY / 256;                       // outputs per thread and plane
+  const int ox = tid % TX, oy = tid / TX;
+  float s0[NO], s1[NO];                                       // sums of planes zi - 1, zi
+#pragma unroll
+  for (int o = 0; o < NO; ++o) s0[o] = s1[o] = 0.f;
+  // three tiles' loads in flight per lane; those of a plane's first three are
+  // issued before the previous plane's sums
+  uint4 a[3][2];
+  auto load3 = [&](int zi, int k0) {
+    const uint4* hp = reinterpret_cast<const uint4*>(H3 + (base + wrap(zi, Z) * plane) * C) + t;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (k0 + k < TPW && warp + 8 * (k0 + k) < OT::NT) {
+        a[k][0] = hp[4ll * off[k0 + k][0]];
+        a[k][1] = hp[4ll * off[k0 + k][1]];
+      }
+  };
+  load3(z0 - 1, 0);
+  for (int zi = z0 - 1; zi <= z1; ++zi) {
+#pragma unroll
+    for (int k0 = 0; k0 < TPW; k0 += 3) {
+      if (k0) load3(zi, k0);
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (k0 + k < TPW && warp + 8 * (k0 + k) < OT::NT) {
+          float* dst = tsm + (warp + 8 * (k0 + k)) * 16 + g;
+          const uint32_t a0[4] = {a[k][0].x, a[k][1].x, a[k][0].y, a[k][1].y};
+          const uint32_t a1[4] = {a[k][0].z, a[k][1].z, a[k][0].w, a[k][1].w};
+#pragma unroll
+          for (int n = 0; n < 4; ++n) {
+            float d[4] = {0.f, 0.f, 0.f, 0.f};
+            const uint32_t b0[2] = {wf[n].x, wf[n].y}, b1[2] = {wf[4 + n].x, wf[4 + n].y};
+            mma_bf16(d, a0, b0);
+            mma_bf16(d, a1, b1);
+            const int tap = 8 * n + 2 * t;
+            if (tap < TAPS) {
+              dst[tap * OT::LD] = d[0];
+              dst[tap * OT::LD + 8] = d[2];
+            }
+            if (tap + 1 < TAPS) {
+              dst[(tap + 1) * OT::LD] = d[1];
+              dst[(tap + 1) * OT::LD + 8] = d[3];
+            }
+          }
+        }
+    }
+    if (zi < z1) load3(zi + 1, 0);
+    __syncthreads();
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+      const int yl = oy + o * (256 / TX);
+      const float* sp = tsm + yl * (TX + 2) + ox;
+      float p[3] = {0.f, s1[o], s0[o]};                       // tap a adds to output plane zi + 1 - a
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int bc = 0; bc < 9; ++bc) p[a] += sp[(a * 9 + bc) * OT::LD + (bc / 3) * (TX + 2) + bc % 3];
+      s1[o] = p[0];
+      s0[o] = p[1];
+      if (zi > z0 && y0 + yl < Y) {
+        const long long gi = base + (zi - 1) * plane + (long long)(y0 + yl) * X + x0 + ox;
+        u0[gi] = ubar[gi] + sig * p[2];
+      }
+    }
+    __syncthreads();
   }
+}
+
+template <int TX>
+static cudaError_t launch_conv_out(const CnnBuffers& w, const float* ubar, float* u0, int X, int Y, int Z, int B,
+                                   double ascale, cudaStream_t s) {
+  const long long cols = (long long)(X / TX) * ((Y + OUT_TY - 1) / OUT_TY);
+  int zc = Z;       // planes per block: at least four waves of three blocks per SM, and at least 8 planes (halo 2 of 10)
+  while (zc > 8 && cols * B * ((Z + zc - 1) / zc) < 4 * 3 * 152) zc = (zc + 1) / 2;
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_conv_out<TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OutTile<TX>::smem);
+  if (e != cudaSuccess) return e;
+  k_conv_out<TX><<<dim3((unsigned)(cols * ((Z + zc - 1) / zc)), B), 256, OutTile<TX>::smem, s>>>(
+      w.H3, w.frag4, ubar, w.sumsq, u0, X, Y, Z, zc, ascale);
+  return cudaGetLastError();
 }
 
 // Weight gradients of the 1-channel layers, as one correlation of a scalar
@@ -575,6 +764,8 @@ __global__ void __launch_bounds__(256) k_conv_out_bwd(const float* __restrict__ 
 // sliding register window, so each point costs 9 shared loads, one 64-byte
 // coalesced load of V and 27 FMAs per lane. The warps' sums are added in the
 // block (fixed order) and written as one float32 partial of 27 x 32 per block.
+// 1/sigma_b takes a float64 root and divide, which every thread computed per
+// segment before (first layer, 64^3 x 8: 480 -> 288 us).
 __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
   const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
@@ -611,6 +802,8 @@ __global__ void __launch_bounds__(256, 3) k_wgrad_1ch(const float* __restrict__ 
 #pragma unroll
   for (int t = 0; t < TAPS; ++t) acc[t] = 0.f;
   const int npw = TW / 8, xs = warp * npw;
+  int sb_of = -1;
+  float scale = 1.f;
   long long r = blockIdx.x;
   if (r < nrows) stage_1ch(sw, S, r, segs, X, Y, Z, TW, P);
   cp_async_commit();
@@ -623,7 +816,10 @@ __global__ void __launch_bounds__(256, 3) k_wgrad_1ch(const float* __restrict__ 
     const int seg = (int)(r % segs);
     const long long q = r / segs;                   // (b, z, y) row index
     const int b = (int)(q / ((long long)Z * Y));
-    const float scale = sumsq ? (float)(1.0 / sqrt(fmax(sumsq[b] / (double)P, 1e-300))) : 1.f;
+    if (sumsq && b != sb_of) {                      // float64 divide and root only where the sample changes
+      scale = (float)(1.0 / sqrt(fmax(sumsq[b] / (double)P, 1e-300)));
+      sb_of = b;
+    }
     const __nv_bfloat16* vrow = V + (q * X + seg * TW + xs) * C + lane;
     float win[9][3];
 #pragma unroll
@@ -659,13 +855,24 @@ __global__ void __launch_bounds__(256, 3) k_wgrad_1ch(const float* __restrict__ 
   }
 }
 
-// out[i] = sum_j part[j][i] (fixed order), j < nparts, i < n.
-__global__ void k_reduce_parts(const float* __restrict__ part, int nparts, int n, float* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// out[i] = sum_j part[j][i] (fixed order), j < nparts, i < n, n a multiple of
+// 32. A block owns 32 columns: warp w sums the parts j = w, w + 8, .. of its
+// columns (coalesced rows of 128 bytes, four in flight), then the eight warps'
+// float64 sums are added in order. One thread per column over all the parts
+// left 4 blocks on a chain of 456 dependent loads (864 columns: 73 -> 15 us).
+__global__ void __launch_bounds__(256) k_reduce_parts(const float* __restrict__ part, int nparts, int n,
+                                                      float* __restrict__ out) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
   double s = 0.0;
-  for (int j = 0; j < nparts; ++j) s += part[(long long)j * n + i];
-  out[i] = (float)s;
+#pragma unroll 4
+  for (int j = w; j < nparts; j += 8) s += part[(long long)j * n + i];
+  red[w][lane] = s;
+  __syncthreads();
+  if (w == 0) {
+    for (int q = 1; q < 8; ++q) s += red[q][lane];
+    out[i] = (float)s;
+  }
 }
 
 // Adam on the float32 master weights.
@@ -687,8 +894,17 @@ __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __re
 
 int cnn_tile(int X) { return X % 64 == 0 ? 64 : 32; }
 
-// two halves of three staged rows each (double-buffered z offsets)
-size_t cnn_conv_smem(int X) { return (size_t)2 * 3 * (cnn_tile(X) + 2) * ROWB; }
+// One 32 -> 32 layer on the warp-level tensor-core kernel.
+static cudaError_t launch_conv_mma(const __nv_bfloat16* in, const uint2* frag, __nv_bfloat16* out,
+                                   const __nv_bfloat16* mask, int X, int Y, int Z, int B, int mode, cudaStream_t s) {
+  const int TX = cnn_tile(X);
+  const size_t sm = (size_t)2 * (CONV_TY + 2) * (TX + 2) * ROWB;   // two z offsets' rows
+  const cudaError_t e = cudaFuncSetAttribute(k_conv_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const dim3 g((unsigned)((X / TX) * ((Y + CONV_TY - 1) / CONV_TY)) * Z, B);
+  k_conv_mma<<<g, TX / 32 * 64, sm, s>>>(in, frag, out, mask, X, Y, Z, TX, mode);
+  return cudaGetLastError();
+}
 
 bool cnn_shape_ok(int X, int Y, int Z) { return X % 32 == 0 && Y >= 3 && Z >= 3; }
 
@@ -696,32 +912,31 @@ cudaError_t cnn_forward(const CnnBuffers& w, const float* ubar, float* u0, const
                         int B, double ascale, cudaStream_t s) {
   const long long P = (long long)X * Y * Z;
   const int TX = cnn_tile(X);
-  const size_t sm = cnn_conv_smem(X);
   cudaError_t e = cudaMemsetAsync(w.sumsq, 0, sizeof(double) * 2 * B + sizeof(double), s);
   if (e != cudaSuccess) return e;
   const dim3 gp((unsigned)((P + 255) / 256 < 2048 ? (P + 255) / 256 : 2048), B);
   k_sumsq<<<gp, 256, 0, s>>>(ubar, P, w.sumsq);
   if (utrue) k_sumsq<<<gp, 256, 0, s>>>(utrue, P, w.sumsq + B);
-  k_conv_in<<<gp, 256, 0, s>>>(ubar, w.sumsq, w.master, w.H1, X, Y, Z);
-  if (sm > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_conv_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-  }
-  const dim3 gc((unsigned)(X / TX) * Y * Z, B);
+  const dim3 g1((unsigned)(P / 512 < 4096 ? (P + 511) / 512 : 4096), B);
+  k_conv_1ch<false><<<g1, 128, kConv1Smem, s>>>(ubar, w.sumsq, w.master, nullptr, w.H1, X, Y, Z);
   if (w.umma2 && conv_tc_shape_ok(X, Y, Z)) {
     if ((e = conv_tc_forward(w.H1, w.umma2, w.H2, nullptr, X, Y, Z, B, 0, w.flag, w.wait_ns, s)) != cudaSuccess ||
         (e = conv_tc_forward(w.H2, w.umma3, w.H3, nullptr, X, Y, Z, B, 0, w.flag, w.wait_ns, s)) != cudaSuccess)
       return e;
   } else {
-    k_conv_mma<<<gc, TX, sm, s>>>(w.H1, w.frag2, w.H2, nullptr, X, Y, Z, TX, 0);
-    k_conv_mma<<<gc, TX, sm, s>>>(w.H2, w.frag3, w.H3, nullptr, X, Y, Z, TX, 0);
+    if ((e = launch_conv_mma(w.H1, w.frag2, w.H2, nullptr, X, Y, Z, B, 0, s)) != cudaSuccess ||
+        (e = launch_conv_mma(w.H2, w.frag3, w.H3, nullptr, X, Y, Z, B, 0, s)) != cudaSuccess)
+      return e;
   }
-  if (sm > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_conv_out_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-  }
-  k_conv_out_mma<<<gc, TX, sm, s>>>(w.H3, w.frag4, ubar, w.sumsq, u0, utrue, w.sumsq + B, w.g, w.sumsq + 2 * B,
-                                    X, Y, Z, B, TX, ascale);
+  if (!utrue)
+    return X % 64 == 0 ? launch_conv_out<64>(w, ubar, u0, X, Y, Z, B, ascale, s)
+                       : launch_conv_out<32>(w, ubar, u0, X, Y, Z, B, ascale, s);
+  const size_t sm = (size_t)10 * (TX + 2) * ROWB;
+  e = cudaFuncSetAttribute(k_conv_out_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const dim3 gc((unsigned)((X / TX) * ((Y + 7) / 8)) * Z, B);
+  k_conv_out_mma<<<gc, 2 * TX, sm, s>>>(w.H3, w.frag4t, ubar, w.sumsq, u0, utrue, w.sumsq + B, w.g, w.sumsq + 2 * B,
+                                        X, Y, Z, B, TX, ascale);
   return cudaGetLastError();
 }
 
@@ -731,14 +946,7 @@ cudaError_t cnn_conv_layer(const CnnBuffers& w, int X, int Y, int Z, int B, cuda
   const bool tc = w.umma2 && conv_tc_shape_ok(X, Y, Z);
   if (tensor_cores) *tensor_cores = tc;
   if (tc) return conv_tc_forward(w.H1, w.umma2, w.H2, nullptr, X, Y, Z, B, 0, w.flag, w.wait_ns, s);
-  const int TX = cnn_tile(X);
-  const size_t sm = cnn_conv_smem(X);
-  if (sm > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_conv_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-  }
-  k_conv_mma<<<dim3((unsigned)(X / TX) * Y * Z, B), TX, sm, s>>>(w.H1, w.frag2, w.H2, nullptr, X, Y, Z, TX, 0);
-  return cudaGetLastError();
+  return launch_conv_mma(w.H1, w.frag2, w.H2, nullptr, X, Y, Z, B, 0, s);
 }
 
 cudaError_t cnn_pack(const CnnBuffers& w, cudaStream_t s) {
@@ -747,7 +955,8 @@ cudaError_t cnn_pack(const CnnBuffers& w, cudaStream_t s) {
   k_pack_frag<<<(n + 255) / 256, 256, 0, s>>>(w.master + kW3, w.frag3, 0);
   k_pack_frag<<<(n + 255) / 256, 256, 0, s>>>(w.master + kW2, w.frag2t, 1);
   k_pack_frag<<<(n + 255) / 256, 256, 0, s>>>(w.master + kW3, w.frag3t, 1);
-  k_pack_frag4<<<(TAPS * 2 * 32 + 255) / 256, 256, 0, s>>>(w.master + kW4, w.frag4);
+  k_pack_frag4<<<1, 256, 0, s>>>(w.master + kW4, w.frag4);
+  k_pack_frag4t<<<(180 * 32 + 255) / 256, 256, 0, s>>>(w.master + kW4, w.frag4t);
   if (w.umma2) {
     cudaError_t e;
     if ((e = conv_tc_pack(w.master + kW2, w.umma2, 0, s)) != cudaSuccess ||
@@ -775,38 +984,36 @@ static size_t wgrad_1ch_smem(int TW) {
 cudaError_t cnn_backward(const CnnBuffers& w, const float* ubar, int X, int Y, int Z, int B, cudaStream_t s) {
   const long long P = (long long)X * Y * Z;
   const int TX = cnn_tile(X);
-  const size_t sm = cnn_conv_smem(X);
-  const dim3 gp((unsigned)((P + 255) / 256 < 2048 ? (P + 255) / 256 : 2048), B);
-  const dim3 gc((unsigned)(X / TX) * Y * Z, B);
   // layer 4
-  k_conv_out_bwd<<<gp, 256, 0, s>>>(w.g, w.master + kW4, w.H3, w.dA, X, Y, Z);
+  const dim3 g1((unsigned)(P / 512 < 4096 ? (P + 511) / 512 : 4096), B);
+  k_conv_1ch<true><<<g1, 128, kConv1Smem, s>>>(w.g, nullptr, w.master + kW4, w.H3, w.dA, X, Y, Z);
   const int TW = wgrad_1ch_tile(X);
   const size_t sm1 = wgrad_1ch_smem(TW);
   k_wgrad_1ch<<<kSmallBlocks, 256, sm1, s>>>(w.g, nullptr, w.H3, w.part, X, Y, Z, B, TW, 1);
-  k_reduce_parts<<<(TAPS * C + 255) / 256, 256, 0, s>>>(w.part, kSmallBlocks, TAPS * C, w.grad + kW4);
+  k_reduce_parts<<<TAPS * C / 32, 256, 0, s>>>(w.part, kSmallBlocks, TAPS * C, w.grad + kW4);
   // layer 3: dW3 from (H2, dZ3); dZ2 = conv^T(dZ3, W3) masked by H2
-  const size_t smw = (size_t)10 * (TX + 2) * ROWB;
+  const size_t smw = (size_t)(WG_H * 3 * (TX + 2) + WG_Z * TX) * ROWB;
   cudaError_t e = cudaFuncSetAttribute(k_wgrad_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw);
   if (e != cudaSuccess) return e;
-  k_wgrad_mma<<<kWgradBlocks, 288, smw, s>>>(w.H2, w.dA, w.part, X, Y, Z, B, TX);
-  k_reduce_parts<<<(TAPS * C * C + 255) / 256, 256, 0, s>>>(w.part, kWgradBlocks, TAPS * C * C, w.grad + kW3);
+  k_wgrad_mma<<<kWgradBlocks, 576, smw, s>>>(w.H2, w.dA, w.part, X, Y, Z, B, TX);
+  k_reduce_parts<<<TAPS * C * C / 32, 256, 0, s>>>(w.part, kWgradBlocks, TAPS * C * C, w.grad + kW3);
   const bool tc = w.umma2 && conv_tc_shape_ok(X, Y, Z);
   if (tc) {
     if ((e = conv_tc_forward(w.dA, w.umma3t, w.dB, w.H2, X, Y, Z, B, 1, w.flag, w.wait_ns, s)) != cudaSuccess) return e;
   } else {
-    k_conv_mma<<<gc, TX, sm, s>>>(w.dA, w.frag3t, w.dB, w.H2, X, Y, Z, TX, 1);
+    if ((e = launch_conv_mma(w.dA, w.frag3t, w.dB, w.H2, X, Y, Z, B, 1, s)) != cudaSuccess) return e;
   }
   // layer 2: dW2 from (H1, dZ2); dZ1 = conv^T(dZ2, W2) masked by H1
-  k_wgrad_mma<<<kWgradBlocks, 288, smw, s>>>(w.H1, w.dB, w.part, X, Y, Z, B, TX);
-  k_reduce_parts<<<(TAPS * C * C + 255) / 256, 256, 0, s>>>(w.part, kWgradBlocks, TAPS * C * C, w.grad + kW2);
+  k_wgrad_mma<<<kWgradBlocks, 576, smw, s>>>(w.H1, w.dB, w.part, X, Y, Z, B, TX);
+  k_reduce_parts<<<TAPS * C * C / 32, 256, 0, s>>>(w.part, kWgradBlocks, TAPS * C * C, w.grad + kW2);
   if (tc) {
     if ((e = conv_tc_forward(w.dB, w.umma2t, w.dA, w.H1, X, Y, Z, B, 1, w.flag, w.wait_ns, s)) != cudaSuccess) return e;
   } else {
-    k_conv_mma<<<gc, TX, sm, s>>>(w.dB, w.frag2t, w.dA, w.H1, X, Y, Z, TX, 1);
+    if ((e = launch_conv_mma(w.dB, w.frag2t, w.dA, w.H1, X, Y, Z, B, 1, s)) != cudaSuccess) return e;
   }
   // layer 1
   k_wgrad_1ch<<<kSmallBlocks, 256, sm1, s>>>(ubar, w.sumsq, w.dA, w.part, X, Y, Z, B, TW, 0);
-  k_reduce_parts<<<(TAPS * C + 255) / 256, 256, 0, s>>>(w.part, kSmallBlocks, TAPS * C, w.grad + kW1);
+  k_reduce_parts<<<TAPS * C / 32, 256, 0, s>>>(w.part, kSmallBlocks, TAPS * C, w.grad + kW1);
   return cudaGetLastError();
 }
 

@@ -15,7 +15,7 @@ constexpr int kW3 = kW2 + 27 * 32 * 32;      // [27][32][32]
 constexpr int kW4 = kW3 + 27 * 32 * 32;      // [27][32]
 constexpr int kCnnWeights = kW4 + 27 * 32;
 constexpr int kSmallBlocks = 456;            // blocks of the 1-channel weight-gradient kernel (3 per SM)
-constexpr int kWgradBlocks = 304;            // blocks of the 32x32 weight-gradient kernel
+constexpr int kWgradBlocks = 152;            // blocks of the 32x32 weight-gradient kernel (1 per SM)
 
 struct CnnBuffers {
   float* master = nullptr;     // weights
@@ -26,7 +26,8 @@ struct CnnBuffers {
   uint2* frag3 = nullptr;
   uint2* frag2t = nullptr;     // flipped, channel-swapped (backward data)
   uint2* frag3t = nullptr;
-  uint2* frag4 = nullptr;      // layer 4 weights as one n8 tile (column 0) in mma fragment order
+  uint2* frag4 = nullptr;      // layer 4 weights, one column per tap, in mma fragment order (k_conv_out)
+  uint2* frag4t = nullptr;     // layer 4 weights, one column per output row, in mma fragment order (training steps)
   __nv_bfloat16* H1 = nullptr; // activations [B][P][32]
   __nv_bfloat16* H2 = nullptr;
   __nv_bfloat16* H3 = nullptr;
