@@ -496,6 +496,13 @@ void set_pass(PassArgs<T>& a, const PassCfg& pc) {
 // Blocks always hold whole warps (the reductions shuffle over full warps).
 int block_threads(const PassCfg& pc) { return (pc.T + 31) / 32 * 32; }
 
+template <typename T>
+cudaError_t launch_with_finish(int kind, int E, dim3 grid, int threads, size_t smem, cudaStream_t s,
+                               const PassArgs<T>& a) {
+  const cudaError_t e = launch_pass<T>(kind, E, grid, threads, smem, s, a);
+  return e != cudaSuccess || !a.defer ? e : launch_finish<T>(a, (int)grid.x, (int)grid.y, threads, s);
+}
+
 template <typename T> void store_args(LaunchRec& r, const PassArgs<T>& a);
 template <> void store_args<float>(LaunchRec& r, const PassArgs<float>& a) { r.af = a; r.f64 = false; }
 template <> void store_args<double>(LaunchRec& r, const PassArgs<double>& a) { r.ad = a; r.f64 = true; }
@@ -504,11 +511,19 @@ template <> void store_args<double>(LaunchRec& r, const PassArgs<double>& a) { r
 // a pass then starts on the fields the previous one finished with, whose
 // vectors and spectra may still be in L2. A field's result does not depend on
 // the order.
+//
+// A dot pass of many blocks leaves its sums and recurrences to a k_finish
+// launch (block_finish); the results are the same either way. kDeferBlocks:
+// below it the ticket costs less than another launch (2-3 us in a graph).
+constexpr unsigned kDeferBlocks = 1000;
+
 template <typename T>
-cudaError_t issue(ad_ctx* ctx, int kind, const PassCfg& pc, cudaStream_t s, const PassArgs<T>& a0) {
+cudaError_t issue(ad_ctx* ctx, int kind, const PassCfg& pc, cudaStream_t s, const PassArgs<T>& a0, int* nl) {
   PassArgs<T> a = a0;
   a.rev = ctx->rev_next;
   ctx->rev_next ^= 1;
+  a.defer = a.ndots > 0 && pc.grid.x * pc.grid.y >= kDeferBlocks;
+  *nl += 1 + a.defer;
   if (ctx->record) {
     LaunchRec r;
     r.kind = kind; r.E = pc.E; r.grid = pc.grid; r.threads = block_threads(pc); r.smem = pc.smem;
@@ -516,7 +531,7 @@ cudaError_t issue(ad_ctx* ctx, int kind, const PassCfg& pc, cudaStream_t s, cons
     ctx->record->push_back(r);
     return cudaSuccess;
   }
-  return launch_pass<T>(kind, pc.E, pc.grid, block_threads(pc), pc.smem, s, a);
+  return launch_with_finish<T>(kind, pc.E, pc.grid, block_threads(pc), pc.smem, s, a);
 }
 
 template <typename T>
@@ -528,12 +543,10 @@ ad_status enqueue_G(ad_ctx* ctx, Plan* p, cudaStream_t s, const Fwd& fw, const F
   a.op = fw.op; a.A = (const T*)fw.A; a.B = (const T*)fw.B;
   a.O1 = (T*)fw.O1; a.O2 = (T*)fw.O2; a.O3 = (T*)fw.O3;
   a.ndots = 0; a.stage = SS_NONE; a.set_cond = 0; a.clear_cond = (fw.clear_cond && c.in_graph) ? 1 : 0;
-  CK(issue<T>(ctx, PK_XFWD, p->xf, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_XFWD, p->xf, s, a, nl));
   if (p->ndim == 3) {
     set_pass(a, p->yf);
-    CK(issue<T>(ctx, PK_YFWD, p->yf, s, a));
-    ++*nl;
+    CK(issue<T>(ctx, PK_YFWD, p->yf, s, a, nl));
   }
   a.clear_cond = 0;
   set_pass(a, p->fl);
@@ -541,20 +554,17 @@ ad_status enqueue_G(ad_ctx* ctx, Plan* p, cudaStream_t s, const Fwd& fw, const F
   a.ndots = fl.op == FI_NONE ? 0 : (fl.op == FI_XGX ? 1 : 3);
   a.stage = fl.stage;
   a.inv_p = 1.0 / (double)p->P;       // Parseval: (a, b) = (1/P) sum_k a_hat conj(b_hat)
-  CK(issue<T>(ctx, PK_FILT, p->fl, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_FILT, p->fl, s, a, nl));
   a.ndots = 0; a.stage = SS_NONE; a.inv_p = 1.0;
   if (p->ndim == 3) {
     set_pass(a, p->yi);
-    CK(issue<T>(ctx, PK_YINV, p->yi, s, a));
-    ++*nl;
+    CK(issue<T>(ctx, PK_YINV, p->yi, s, a, nl));
   }
   set_pass(a, p->xi);
   a.op = iv.op; a.A = (const T*)iv.A; a.B = (const T*)iv.B; a.C = (const T*)iv.C;
   a.O1 = (T*)iv.O1; a.O2 = (T*)iv.O2; a.O3 = nullptr;
   a.ndots = iv.ndots; a.stage = iv.stage; a.set_cond = (iv.set_cond && c.in_graph) ? 1 : 0;
-  CK(issue<T>(ctx, PK_XINV, p->xi, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_XINV, p->xi, s, a, nl));
   return AD_OK;
 }
 
@@ -578,17 +588,14 @@ ad_status enqueue_fwd_transform(ad_ctx* ctx, Plan* p, cudaStream_t s, const void
   PassArgs<T> a = base_args<T>(p, c0);
   set_pass(a, p->xf);
   a.op = XF_COPY; a.A = (const T*)x;
-  CK(issue<T>(ctx, PK_XFWD, p->xf, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_XFWD, p->xf, s, a, nl));
   if (p->ndim == 3) {
     set_pass(a, p->yf);
-    CK(issue<T>(ctx, PK_YFWD, p->yf, s, a));
-    ++*nl;
+    CK(issue<T>(ctx, PK_YFWD, p->yf, s, a, nl));
   }
   set_pass(a, p->fl);
   a.O1 = (T*)out;
-  CK(issue<T>(ctx, PK_LFWD, p->fl, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_LFWD, p->fl, s, a, nl));
   return AD_OK;
 }
 
@@ -599,18 +606,15 @@ ad_status enqueue_inv_transform(ad_ctx* ctx, Plan* p, cudaStream_t s, const void
   PassArgs<T> a = base_args<T>(p, c0);
   set_pass(a, p->fl);
   a.A = (const T*)hat;
-  CK(issue<T>(ctx, PK_LINV, p->fl, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_LINV, p->fl, s, a, nl));
   a.A = nullptr;
   if (p->ndim == 3) {
     set_pass(a, p->yi);
-    CK(issue<T>(ctx, PK_YINV, p->yi, s, a));
-    ++*nl;
+    CK(issue<T>(ctx, PK_YINV, p->yi, s, a, nl));
   }
   set_pass(a, p->xi);
   a.op = XI_STORE; a.O1 = (T*)x;
-  CK(issue<T>(ctx, PK_XINV, p->xi, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_XINV, p->xi, s, a, nl));
   return AD_OK;
 }
 
@@ -630,8 +634,7 @@ ad_status enqueue_spec(ad_ctx* ctx, Plan* p, cudaStream_t s, const Spec& sp, con
   a.inv_p = 1.0 / (double)p->P;        // Parseval
   a.clear_cond = (sp.clear_cond && c.in_graph) ? 1 : 0;
   a.set_cond = (sp.set_cond && c.in_graph) ? 1 : 0;
-  CK(issue<T>(ctx, PK_SPEC, p->sp, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_SPEC, p->sp, s, a, nl));
   return AD_OK;
 }
 
@@ -731,8 +734,7 @@ ad_status enqueue_sten(ad_ctx* ctx, Plan* p, cudaStream_t s, const void* r, void
   a.op = 0; a.A = (const T*)r; a.O1 = (T*)z;
   a.ndots = 1; a.stage = SS_PCG_RHO; a.set_cond = 0;
   a.clear_cond = (clear_cond && c.in_graph) ? 1 : 0;
-  CK(issue<T>(ctx, PK_STEN, p->sn, s, a));
-  ++*nl;
+  CK(issue<T>(ctx, PK_STEN, p->sn, s, a, nl));
   return AD_OK;
 }
 
@@ -969,8 +971,8 @@ double time_kind(ad_ctx* ctx, Plan* p, int method, int kind, int reps) {
     r.af.force = r.ad.force = 1;
     r.af.stage = r.ad.stage = SS_NONE;
     r.af.set_cond = r.ad.set_cond = r.af.clear_cond = r.ad.clear_cond = 0;
-    auto go = [&]() { return r.f64 ? launch_pass<double>(r.kind, r.E, r.grid, r.threads, r.smem, nullptr, r.ad)
-                                    : launch_pass<float>(r.kind, r.E, r.grid, r.threads, r.smem, nullptr, r.af); };
+    auto go = [&]() { return r.f64 ? launch_with_finish<double>(r.kind, r.E, r.grid, r.threads, r.smem, nullptr, r.ad)
+                                    : launch_with_finish<float>(r.kind, r.E, r.grid, r.threads, r.smem, nullptr, r.af); };
     cudaError_t e = go();
     if (e == cudaSuccess) e = cudaEventRecord(e0, nullptr);
     for (int i = 0; i < reps && e == cudaSuccess; ++i) e = go();
@@ -1300,6 +1302,7 @@ ad_status merge_multi(ad_ctx* ctx, BatchedEntry& be, std::vector<std::vector<Lau
         a.vgy = (int)rs[g]->grid.y;
         a.vbd = rs[g]->threads;
         a.ms = ms;
+        a.defer = 0;
         if (a.clear_cond) {
           a.clear_cond = (first_clear && !cleared) ? 1 : 0;
           cleared = true;
@@ -1628,8 +1631,8 @@ ad_status ad_time_pass(ad_ctx* ctx, const ad_grid* grid, int batch, ad_method me
     cudaError_t err = cudaSuccess;
     for (size_t i = first; i < last && err == cudaSuccess; ++i) {
       const LaunchRec& q = rec[i];
-      err = q.f64 ? launch_pass<double>(q.kind, q.E, q.grid, q.threads, q.smem, st, q.ad)
-                  : launch_pass<float>(q.kind, q.E, q.grid, q.threads, q.smem, st, q.af);
+      err = q.f64 ? launch_with_finish<double>(q.kind, q.E, q.grid, q.threads, q.smem, st, q.ad)
+                  : launch_with_finish<float>(q.kind, q.E, q.grid, q.threads, q.smem, st, q.af);
     }
     return err;
   };

@@ -129,6 +129,7 @@ struct PassArgs {
   SolveConfig cfg;
   double* part;              // [batch][gridDim.x][4] block partial dots
   unsigned* ticket;          // [0] fields done, [1] loop passes, [2 + f] blocks of field f
+  int defer;                 // the dots are finished by a k_finish launch that follows
   int stage;                 // ScalarStage run by the last block
   int set_cond;              // last block sets the graph's while-condition
   cudaGraphConditionalHandle cond;

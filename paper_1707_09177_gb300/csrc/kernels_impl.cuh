@@ -57,6 +57,12 @@ cudaError_t launch_pass(int kind, int E, dim3 grid, int threads, size_t smem, cu
 }
 
 template <typename T>
+cudaError_t launch_finish(const PassArgs<T>& a, int nblk, int batch, int threads, cudaStream_t s) {
+  k_finish<T><<<batch, threads, 0, s>>>(a, nblk);
+  return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t launch_cg_finish(T* u, const T* p, const FieldState* st, long long P, int batch, cudaStream_t s) {
   const long long n4 = P / 4;
   int blocks = (int)((n4 + 255) / 256);
@@ -111,6 +117,7 @@ template cudaError_t launch_hist<GAD_REAL>(const GAD_REAL*, long long, double, d
                                            cudaStream_t);
 template cudaError_t launch_curl<GAD_REAL>(const void*, void*, int, int, int, long long, int, int, cudaStream_t);
 template cudaError_t launch_pass<GAD_REAL>(int, int, dim3, int, size_t, cudaStream_t, const PassArgs<GAD_REAL>&);
+template cudaError_t launch_finish<GAD_REAL>(const PassArgs<GAD_REAL>&, int, int, int, cudaStream_t);
 template cudaError_t launch_cg_finish<GAD_REAL>(GAD_REAL*, const GAD_REAL*, const FieldState*, long long, int,
                                                 cudaStream_t);
 

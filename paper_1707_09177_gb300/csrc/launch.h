@@ -29,6 +29,10 @@ template <typename T>
 cudaError_t launch_multi(int kind, int E, int blocks, int threads, size_t smem, cudaStream_t s,
                          const PassArgs<T>* args, const int* start, int ngroups);
 
+// Ends a deferred dot pass of `nblk` blocks per field and `batch` fields.
+template <typename T>
+cudaError_t launch_finish(const PassArgs<T>& a, int nblk, int batch, int threads, cudaStream_t s);
+
 template <typename T>
 cudaError_t launch_cg_finish(T* u, const T* p, const FieldState* st, long long P, int batch, cudaStream_t s);
 

@@ -259,107 +259,71 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Block reduction of up to three dots into a per-block partial, then two
-// arrival tickets. ticket[2 + f] counts the blocks of field f: the last one
-// to arrive sums that field's partials in a fixed order (deterministic for a
-// fixed launch shape) and runs the field's scalar update at once, while
-// other fields' blocks are still running. ticket[0] counts finished fields:
-// the last one sets the graph's loop condition. ticket[1] counts loop passes
-// of the current solve (reset by the initial-residual pass).
+// t[d] += the partials b = tid, tid + nthr, .. of dot d, eight loads in flight.
+template <int ND>
+__device__ __forceinline__ void sum_partials(const double* pf, int nblk, int tid, int nthr, double* t) {
+  int b = tid;
+  for (; b + 7 * nthr < nblk; b += 8 * nthr) {
+    double v[8][ND];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+      for (int d = 0; d < ND; ++d) v[k][d] = __ldcg(pf + (long long)(b + k * nthr) * 4 + d);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+      for (int d = 0; d < ND; ++d) t[d] += v[k][d];
+  }
+  for (; b < nblk; b += nthr)
+#pragma unroll
+    for (int d = 0; d < ND; ++d) t[d] += __ldcg(pf + (long long)b * 4 + d);
+}
+
+// The sum of a field's block partials in a fixed order (deterministic for a
+// fixed launch shape; the order of a `nthr`-thread block), the field's scalar
+// update, and, by the last field to get here, the graph's loop condition.
+// ticket[0] counts the fields done, ticket[1] the loop passes of the current
+// solve (reset by the initial-residual pass). Run by one whole block.
 template <typename T>
-__device__ void block_finish(const PassArgs<T>& a, const Acc<T>* acc, int f, bool act, const VBlock& vb) {
+__device__ __forceinline__ void finish_field(const PassArgs<T>& a, int f, bool act, int nblk, int nfields_launch,
+                                             int nthr) {
   __shared__ double red[32][3];
-  __shared__ int last_field;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // the block size of the pass's own launch shape (a k_multi block may be
-  // larger: its extra threads hold no terms), so that the reduction order,
-  // and with it every rounding, is the same in both kinds of launch
-  const int nthr = a.vbd ? a.vbd : (int)blockDim.x;
-  const int nw = (nthr + 31) >> 5;
-  const int nblk = vb.nx;
-  if (act) {
-    if constexpr (sizeof(T) == 4) {
-      // float32 dots: the thread's compensated pair, reduced as float pairs
-      __shared__ float2 redf[32][3];
-      float2 v[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const float hi = acc[d].s + acc[d].c;
-        v[d] = warp_sum(make_float2(hi, acc[d].c - (hi - acc[d].s)));
-      }
-      if (lane == 0) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) redf[warp][d] = v[d];
-      }
-      __syncthreads();
-      if (warp == 0) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          float2 t = lane < nw ? redf[lane][d] : make_float2(0.f, 0.f);
-          t = warp_sum(t);
-          if (lane == 0) a.part[((long long)f * nblk + vb.x) * 4 + d] = ((double)t.x + (double)t.y) * a.inv_p;
-        }
-      }
-    } else {
-      double v[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) v[d] = warp_sum(acc[d].value());
-      if (lane == 0) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) red[warp][d] = v[d];
-      }
-      __syncthreads();
-      if (warp == 0) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          double t = lane < nw ? red[lane][d] : 0.0;
-          t = warp_sum(t);
-          if (lane == 0) a.part[((long long)f * nblk + vb.x) * 4 + d] = t * a.inv_p;
-        }
-      }
-    }
-  }
-  if (tid == 0) {
-    __threadfence();
-    const unsigned prev = atomicAdd(a.ticket + 2 + f, 1u);
-    last_field = (prev == (unsigned)nblk - 1u);
-  }
-  __syncthreads();
-  if (!last_field) return;
-  __threadfence();
+  const int nw = (nthr + 31) >> 5, nd = a.ndots;
   FieldState& s = a.st[f];
   if (act) {                    // act is the field's flag: every block of f saw the same value
     double t[3] = {0.0, 0.0, 0.0};
     const double* pf = a.part + (long long)f * nblk * 4;
-    for (int b = tid; b < nblk && tid < nthr; b += nthr) {
-#pragma unroll
-      for (int d = 0; d < 3; ++d) t[d] += __ldcg(pf + (long long)b * 4 + d);
+    if (tid < nthr) {
+      if (nd == 1) sum_partials<1>(pf, nblk, tid, nthr, t);
+      else if (nd == 2) sum_partials<2>(pf, nblk, tid, nthr, t);
+      else sum_partials<3>(pf, nblk, tid, nthr, t);
     }
 #pragma unroll
-    for (int d = 0; d < 3; ++d) t[d] = warp_sum(t[d]);
+    for (int d = 0; d < 3; ++d)
+      if (d < nd) t[d] = warp_sum(t[d]);
     __syncthreads();
     if (lane == 0) {
 #pragma unroll
-      for (int d = 0; d < 3; ++d) red[warp][d] = t[d];
+      for (int d = 0; d < 3; ++d)
+        if (d < nd) red[warp][d] = t[d];
     }
     __syncthreads();
     if (tid == 0) {
-      double tot[3];
+      double tot[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        tot[d] = 0.0;
-        for (int q = 0; q < nw; ++q) tot[d] += red[q][d];
-      }
+      for (int d = 0; d < 3; ++d)
+        if (d < nd)
+          for (int q = 0; q < nw; ++q) tot[d] += red[q][d];
       scalar_update(a.stage, s, tot, a.cfg, f);
     }
   }
   if (tid == 0) {
-    a.ticket[2 + f] = 0u;
     __threadfence();
     // fields done: those of this launch, or, when one sequence of launches
     // serves several shape groups, those of every group (MultiState)
     unsigned* done = a.ms ? a.ms->ticket : a.ticket;
-    const unsigned nfields = a.ms ? (unsigned)a.ms->nfields : (unsigned)vb.ny;
+    const unsigned nfields = a.ms ? (unsigned)a.ms->nfields : (unsigned)nfields_launch;
     const unsigned prevg = atomicAdd(done, 1u);
     if (prevg == nfields - 1u) {                          // every field is reduced
       __threadfence();
@@ -382,6 +346,75 @@ __device__ void block_finish(const PassArgs<T>& a, const Acc<T>* acc, int f, boo
       done[0] = 0u;
     }
   }
+}
+
+// Block reduction of up to three dots into a per-block partial. Launches of
+// few blocks then take an arrival ticket (ticket[2 + f] counts the blocks of
+// field f) and the last block of a field runs finish_field at once. In a launch
+// of many blocks (`defer`) the fence in front of a ticket is what costs: it
+// waits for the SM's stores in flight while the block keeps its slot, one
+// block after the other on an SM (one 512^3 field: the filter pass with three
+// dots took 116 us longer than without at 16,448 blocks, 655 us longer at
+// 65,792; counters on lines of their own change nothing). Those leave
+// finish_field to a small kernel of its own (k_finish): inverse x pass with one
+// dot 379 -> 337 us (512^3), 217 -> 210 us (2048^2 x 16), filter pass with three
+// dots 193 -> 176 us (2048^2 x 16).
+template <typename T>
+__device__ void block_finish(const PassArgs<T>& a, const Acc<T>* acc, int f, bool act, const VBlock& vb) {
+  __shared__ double red[32][3];
+  __shared__ int last_field;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the block size of the pass's own launch shape (a k_multi block may be
+  // larger: its extra threads hold no terms), so that the reduction order,
+  // and with it every rounding, is the same in both kinds of launch
+  const int nthr = a.vbd ? a.vbd : (int)blockDim.x;
+  const int nw = (nthr + 31) >> 5;
+  const int nblk = vb.nx;
+  const int nd = a.ndots;
+  if (act) {
+    // warp sums, then warp d adds the warps' sums of dot d
+    double* part = a.part + ((long long)f * nblk + vb.x) * 4;
+    if constexpr (sizeof(T) == 4) {
+      // float32 dots: the thread's compensated pair, reduced as float pairs
+      __shared__ float2 redf[32][3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+        if (d < nd) {
+          const float hi = acc[d].s + acc[d].c;
+          const float2 v = warp_sum(make_float2(hi, acc[d].c - (hi - acc[d].s)));
+          if (lane == 0) redf[warp][d] = v;
+        }
+      __syncthreads();
+      for (int d = warp; d < nd; d += nw) {
+        const float2 t = warp_sum(lane < nw ? redf[lane][d] : make_float2(0.f, 0.f));
+        if (lane == 0) part[d] = ((double)t.x + (double)t.y) * a.inv_p;
+      }
+    } else {
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+        if (d < nd) {
+          const double v = warp_sum(acc[d].value());
+          if (lane == 0) red[warp][d] = v;
+        }
+      __syncthreads();
+      for (int d = warp; d < nd; d += nw) {
+        const double t = warp_sum(lane < nw ? red[lane][d] : 0.0);
+        if (lane == 0) part[d] = t * a.inv_p;
+      }
+    }
+    if (nd > 1) __syncthreads();             // the partials of warps 1, 2 precede the ticket below
+  }
+  if (a.defer) return;
+  if (tid == 0) {
+    __threadfence();
+    const unsigned prev = atomicAdd(a.ticket + 2 + f, 1u);
+    last_field = (prev == (unsigned)nblk - 1u);
+    if (last_field) a.ticket[2 + f] = 0u;
+  }
+  __syncthreads();
+  if (!last_field) return;
+  __threadfence();
+  finish_field(a, f, act, nblk, vb.ny, nthr);
 }
 
 template <typename T>
@@ -1076,6 +1109,14 @@ __global__ void GAD_BOUNDS(T, E) k_multi(const PassArgs<T>* __restrict__ args, c
   else if constexpr (KIND == 2) filt_body<T, E>(sa, vb);
   else if constexpr (KIND == 3) yfwd_body<T, E>(sa, vb);
   else if constexpr (KIND == 4) yinv_body<T, E>(sa, vb);
+}
+
+// The end of a deferred dot pass: one block per field, the block size of the
+// pass, `nblk` partials per field.
+template <typename T>
+__global__ void __launch_bounds__(256) k_finish(const __grid_constant__ PassArgs<T> a, int nblk) {
+  const int f = blockIdx.x;
+  finish_field(a, f, a.st[f].active != 0 || a.force, nblk, (int)gridDim.x, (int)blockDim.x);
 }
 
 // u += alpha p for fields whose last CG pass still owes it (Algorithm 3,
