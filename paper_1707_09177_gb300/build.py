@@ -1,6 +1,6 @@
 """Builds the CUDA library libgad.so in-tree for sm_103a with nvcc.
 
-The translation units (host driver, float32 and float64 pass kernels, the
+The translation units (host driver, pass kernels per precision and element count, the
 multi-group pass kernels of batched solves, the allocation-free filter, the
 learned guess's warp-level and tcgen05 kernels) compile in parallel; the result is linked into
 paper_1707_09177_gb300/libgad.so next to this file.
@@ -19,7 +19,14 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgad.so")
-SOURCES = ["api.cu", "kernels_f32.cu", "kernels_f64.cu", "kernels_multi.cu", "noalloc.cu", "cnn.cu", "conv_tc.cu"]
+# (source, defines): the pass kernels are one unit per precision and per-thread
+# element count, the longest to compile first
+SOURCES = ([("kernels_e.cu", ("GAD_REAL=float", "GAD_E=16")), ("kernels_multi.cu", ("GAD_E=16",))]
+           + [("kernels_e.cu", ("GAD_REAL=%s" % t, "GAD_E=%d" % e)) for t in ("float", "double") for e in (24, 16, 12, 4)
+              if (t, e) != ("float", 16)]
+           + [("kernels_multi.cu", ("GAD_E=%d" % e,)) for e in (24, 12, 4)]
+           + [("kernels_fused.cu", ("GAD_LONG=%d" % g,)) for g in (1, 0)]
+           + [(f, ()) for f in ("api.cu", "kernels_f32.cu", "kernels_f64.cu", "noalloc.cu", "cnn.cu", "conv_tc.cu")])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -36,8 +43,10 @@ def _flags():
 
 
 def _compile(src, verbose):
-    obj = os.path.join(BUILD, os.path.splitext(src)[0] + ".o")
-    cmd = [_nvcc()] + _flags() + ["-c", os.path.join(CSRC, src), "-o", obj]
+    src, defines = src
+    name = "_".join([os.path.splitext(src)[0]] + [d.split("=")[1] for d in defines])
+    obj = os.path.join(BUILD, name + ".o")
+    cmd = [_nvcc()] + _flags() + ["-D" + d for d in defines] + ["-c", os.path.join(CSRC, src), "-o", obj]
     if verbose:
         cmd.insert(1, "-Xptxas=-v")
     r = subprocess.run(cmd, capture_output=True, text=True)
@@ -53,7 +62,7 @@ def build(verbose=False, force=False):
     if (not force and os.path.exists(LIB)
             and os.path.getmtime(LIB) > max(os.path.getmtime(d) for d in deps)):
         return LIB
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with ThreadPoolExecutor(max_workers=min(len(SOURCES), os.cpu_count() or 8)) as ex:
         results = list(ex.map(lambda s: _compile(s, verbose), SOURCES))
     if verbose:
         for _, log in results:

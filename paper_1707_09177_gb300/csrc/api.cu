@@ -227,9 +227,9 @@ ad_status get_table(ad_ctx* ctx, long long L, bool f64, const void** out) {
 }
 
 // The tile shape of a pass (plan.h) copied into its launch configuration.
-bool choose_tile(int L, int E, int slots, int div, size_t csize, PassCfg& pc) {
+bool choose_pass(int L, int slots, int div, long long nseq, bool transposed, size_t csize, PassCfg& pc, int want_T) {
   TileShape ts;
-  if (!gad::choose_tile(L, E, slots, div, csize, ts)) return false;
+  if (!gad::choose_pass(L, slots, div, nseq, transposed, csize, ts, want_T)) return false;
   pc.E = ts.E;
   pc.W = ts.W;
   pc.T = ts.T;
@@ -307,33 +307,43 @@ ad_status get_plan(ad_ctx* ctx, const ad_grid* g, int batch, Plan** out) {
   p->twx = tx;                                  // the real-to-complex split of the x passes
   const int M = p->nx / 2;
   const int Lf = p->ndim == 3 ? p->nz : p->ny;
-  const void *px = nullptr, *pf = nullptr, *pfi = nullptr, *py = nullptr;
-  if ((s = get_plan_table(ctx, M, pick_E(M), false, p->f64, &px)) != AD_OK ||
-      (s = get_plan_table(ctx, Lf, pick_E(Lf), false, p->f64, &pf)) != AD_OK ||
-      (s = get_plan_table(ctx, Lf, pick_E(Lf), true, p->f64, &pfi)) != AD_OK ||
-      (p->ndim == 3 && (s = get_plan_table(ctx, p->ny, pick_E(p->ny), false, p->f64, &py)) != AD_OK)) {
+  const int nseq = p->ndim == 3 ? p->kxn * p->ny : p->kxn;
+  const long long nrow = (long long)p->ny * p->nz;
+  // x passes: complex length M (packed real rows); filter pass along the last axis; 3D y passes
+  // Block sizes that measured fastest (us, one launch): forward x pass with
+  // few rows per block (512^3: 469 at 256 threads, 457 at 128, 441 at 64; with
+  // 12 elements per thread 288^3 x 3: 287 at 64, 266 at 128), filter pass at 128
+  // threads (2048^2 x 16: 155 -> 139, 512^3: 284 -> 267), inverse x and y passes
+  // at 256 (512^3: inverse x 337 against 344 at 128, y 211 against 225).
+  bool ok = choose_pass(M, M + 1, pow2_part(p->ny), nrow, true, cs, p->xf, M % 3 == 0 ? 128 : 64);
+  ok = ok && choose_pass(M, M + 1, pow2_part(p->ny), nrow, true, cs, p->xi, 256);
+  ok = ok && choose_pass(Lf, Lf, 0, nseq, false, cs, p->fl, 128);
+  ok = ok && (p->ndim != 3 ||
+              choose_pass(p->ny, p->ny, pow2_part(p->nz), (long long)p->kxn * p->nz, true, cs, p->yf, 256));
+  if (!ok) { delete p; return fail(ctx, AD_ERR_ARG, "no tiling for this grid"); }
+  const void *px = nullptr, *pxi = nullptr, *pf = nullptr, *pfi = nullptr, *py = nullptr;
+  const int ex = plan_E(M, p->xf.E, cs), exi = plan_E(M, p->xi.E, cs), ef = plan_E(Lf, p->fl.E, cs), ey = plan_E(p->ny, p->yf.E, cs);
+  if ((s = get_plan_table(ctx, M, ex, false, p->f64, &px)) != AD_OK ||
+      (s = get_plan_table(ctx, M, exi, false, p->f64, &pxi)) != AD_OK ||
+      (s = get_plan_table(ctx, Lf, ef, false, p->f64, &pf)) != AD_OK ||
+      (s = get_plan_table(ctx, Lf, ef, true, p->f64, &pfi)) != AD_OK ||
+      (p->ndim == 3 && (s = get_plan_table(ctx, p->ny, ey, false, p->f64, &py)) != AD_OK)) {
     delete p;
     return s;
   }
-  bool ok = true;
-  // x passes: complex length M (packed real rows)
-  ok = ok && choose_tile(M, pick_E(M), M + 1, pow2_part(p->ny), cs, p->xf);
-  ok = ok && make_fft(M, p->xf.E, px, p->xf.fft);
-  p->xf.rcp_a = 1.0f / (float)(p->nx / 4);
-  p->xf.rcp_b = 1.0f / (float)(M / 2 + 1);
-  p->xf.grid = dim3(p->ny * p->nz / std::max(p->xf.W, 1), batch);
-  p->xi = p->xf;
-  // filter pass along the last axis
-  const int nseq = p->ndim == 3 ? p->kxn * p->ny : p->kxn;
-  ok = ok && choose_tile(Lf, pick_E(Lf), Lf, 0, cs, p->fl);
-  ok = ok && make_fft(Lf, p->fl.E, pf, p->fl.fft);
-  ok = ok && make_fft(Lf, p->fl.E, pfi, p->fl.fft_inv, true);
+  ok = make_fft(M, ex, px, p->xf.fft) && make_fft(M, exi, pxi, p->xi.fft);
+  for (PassCfg* x : {&p->xf, &p->xi}) {
+    x->rcp_a = 1.0f / (float)(p->nx / 4);
+    x->rcp_b = 1.0f / (float)(M / 2 + 1);
+    x->grid = dim3(p->ny * p->nz / x->W, batch);
+  }
+  ok = ok && make_fft(Lf, ef, pf, p->fl.fft);
+  ok = ok && make_fft(Lf, ef, pfi, p->fl.fft_inv, true);
   p->fl.rcp_a = 1.0f / (float)(Lf / 2);
   p->fl.rcp_b = 1.0f / (float)Lf;
   p->fl.grid = dim3((nseq + std::max(p->fl.W, 1) - 1) / std::max(p->fl.W, 1), batch);
   if (p->ndim == 3) {
-    ok = ok && choose_tile(p->ny, pick_E(p->ny), p->ny, pow2_part(p->nz), cs, p->yf);
-    ok = ok && make_fft(p->ny, p->yf.E, py, p->yf.fft);
+    ok = ok && make_fft(p->ny, ey, py, p->yf.fft);
     p->yf.rcp_a = 1.0f / (float)(p->ny / 2);
     p->yf.rcp_b = 1.0f / (float)p->ny;
     p->yf.grid = dim3(p->kxn * (p->nz / std::max(p->yf.W, 1)), batch);
@@ -935,11 +945,12 @@ struct TileSlot {
 };
 
 void set_tile(const Plan* p, PassCfg& pc, int kind, int L, int slots, int W) {
-  const int ld = tile_ld(slots);
+  const size_t cs = p->f64 ? 16 : 8;
+  const int ld = kind == PK_FILT ? tile_ld(slots) : transposed_ld(tile_ld(slots), W, cs);
   pc.W = W;
   pc.T = (int)((long long)W * L / pc.E);
   pc.ld = ld;
-  pc.smem = (size_t)W * ld * (p->f64 ? 16 : 8);
+  pc.smem = (size_t)W * ld * cs;
   const int nseq = p->ndim == 3 ? p->kxn * p->ny : p->kxn;
   switch (kind) {
     case PK_XFWD: case PK_XINV: pc.grid = dim3(p->ny * p->nz / W, p->batch); break;
@@ -1036,7 +1047,7 @@ ad_status autotune_plan(ad_ctx* ctx, Plan* p, int method, int reps) {
       const long long tot = (long long)W * sl.L;
       if (tot % sl.pc->E != 0) continue;
       const long long T = tot / sl.pc->E;
-      const int ld = tile_ld(sl.slots);
+      const int ld = transposed_ld(tile_ld(sl.slots), W, cs);
       if (T < 32 || T > 256 || (size_t)W * ld * cs > 100 * 1024) continue;
       PassCfg trial = *sl.pc;
       set_tile(p, trial, sl.kind, sl.L, sl.slots, W);

@@ -17,6 +17,7 @@
 #include <stdint.h>
 
 #include "args.h"
+#include "plan.h"
 
 namespace gad {
 
@@ -130,11 +131,44 @@ template <bool INV, typename C> __device__ __forceinline__ void dft16(C* a) {
   }
 }
 
+// 6 = 2 x 3 and 12 = 4 x 3 points by the prime-factor map (no twiddles between
+// the factors): input n = (R/3) n1 + 3 n2 (mod R) and output k with k = k1
+// (mod 3), k = k2 (mod R/3).
+template <bool INV, typename C> __device__ __forceinline__ void dft6(C* a) {
+  C x0 = a[0], x1 = a[2], x2 = a[4], y0 = a[3], y1 = a[5], y2 = a[1];
+  dft3<INV>(x0, x1, x2);
+  dft3<INV>(y0, y1, y2);
+  dft2<INV>(x0, y0);
+  dft2<INV>(x1, y1);
+  dft2<INV>(x2, y2);
+  // (k1, k2) -> k = 4 k1 + 3 k2 (mod 6)
+  a[0] = x0; a[3] = y0; a[4] = x1; a[1] = y1; a[2] = x2; a[5] = y2;
+}
+
+template <bool INV, typename C> __device__ __forceinline__ void dft12(C* a) {
+  C v[3][4];
+#pragma unroll
+  for (int n2 = 0; n2 < 4; ++n2) {
+    v[0][n2] = a[(3 * n2) % 12];
+    v[1][n2] = a[(4 + 3 * n2) % 12];
+    v[2][n2] = a[(8 + 3 * n2) % 12];
+    dft3<INV>(v[0][n2], v[1][n2], v[2][n2]);
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    dft4<INV>(v[k1][0], v[k1][1], v[k1][2], v[k1][3]);
+#pragma unroll
+    for (int k2 = 0; k2 < 4; ++k2) a[(4 * k1 + 9 * k2) % 12] = v[k1][k2];
+  }
+}
+
 template <int R, bool INV, typename C> __device__ __forceinline__ void dft(C* v) {
   if constexpr (R == 2) dft2<INV>(v[0], v[1]);
   else if constexpr (R == 3) dft3<INV>(v[0], v[1], v[2]);
   else if constexpr (R == 4) dft4<INV>(v[0], v[1], v[2], v[3]);
+  else if constexpr (R == 6) dft6<INV>(v);
   else if constexpr (R == 8) dft8<INV>(v);
+  else if constexpr (R == 12) dft12<INV>(v);
   else if constexpr (R == 16) dft16<INV>(v);
 }
 
@@ -177,16 +211,15 @@ __device__ __forceinline__ int run_stride(int st) {
 // stage. `mid_barrier` separates the loads from the writes when both touch
 // the same shared-memory tile.
 //
-// LRC and NSC, when nonzero, are L/R and ns as compile-time constants (powers
-// of two): the sequence and sub-transform indices become shifts and masks and
-// the shared-memory runs get immediate offsets. They must equal the plan's
+// LRC and NSC, when nonzero, are L/R and ns as compile-time constants: the
+// sequence and sub-transform indices become shifts and masks (or
+// multiplications) and the shared-memory runs get immediate offsets. They must equal the plan's
 // values (fft_run_fixed checks the plan before taking that path).
 template <typename C, int E, int R, bool INV, int LRC = 0, int NSC = 0, class Load, class Emit>
 __device__ __forceinline__ void stage_io(int L, const FftStage& sg, const C* __restrict__ tw, int tid, int nthr,
                                          Load& load, Emit& emit, bool mid_barrier) {
   constexpr int NB = E / R;
   static_assert(NB * R == E, "radix must divide the per-thread element count");
-  static_assert((LRC & (LRC - 1)) == 0 && (NSC & (NSC - 1)) == 0, "constant strides are powers of two");
   const int lr = LRC ? LRC : L / R;
   const int ns = NSC ? NSC : sg.ns;
   C v[NB][R];
@@ -267,7 +300,6 @@ __device__ __forceinline__ void stage_filter(int L, const FftStage& sg, const C*
                                              Load& load, Mul& mul, Emit& emit, bool mid_barrier) {
   constexpr int NB = E / R;
   static_assert(NB * R == E, "radix must divide the per-thread element count");
-  static_assert((LRC & (LRC - 1)) == 0, "constant strides are powers of two");
   const int lr = LRC ? LRC : L / R;
   C v[NB][R];
   int wrow[NB], jj[NB];
@@ -344,6 +376,9 @@ __device__ __forceinline__ FftStage stage_at(const FftPlan& p, int q) {
   }
 }
 
+// The radices 6 and 12 occur in float32 plans at 12 elements per thread only.
+template <typename C, int E> constexpr bool fused = sizeof(C) == 8 && E == 12;
+
 // Runtime radix -> compile-time stage.
 template <typename C, int E, bool INV, class Load, class Emit>
 __device__ __forceinline__ void stage_dispatch(int L, const FftStage& sg, const C* __restrict__ tw, int tid, int nthr,
@@ -352,7 +387,9 @@ __device__ __forceinline__ void stage_dispatch(int L, const FftStage& sg, const 
     case 2: if constexpr (E % 2 == 0) stage_io<C, E, 2, INV>(L, sg, tw, tid, nthr, load, emit, mid_barrier); break;
     case 3: if constexpr (E % 3 == 0) stage_io<C, E, 3, INV>(L, sg, tw, tid, nthr, load, emit, mid_barrier); break;
     case 4: if constexpr (E % 4 == 0) stage_io<C, E, 4, INV>(L, sg, tw, tid, nthr, load, emit, mid_barrier); break;
+    case 6: if constexpr (fused<C, E>) stage_io<C, E, 6, INV>(L, sg, tw, tid, nthr, load, emit, mid_barrier); break;
     case 8: if constexpr (E % 8 == 0) stage_io<C, E, 8, INV>(L, sg, tw, tid, nthr, load, emit, mid_barrier); break;
+    case 12: if constexpr (fused<C, E>) stage_io<C, E, 12, INV>(L, sg, tw, tid, nthr, load, emit, mid_barrier); break;
     case 16: if constexpr (E % 16 == 0) stage_io<C, E, 16, INV>(L, sg, tw, tid, nthr, load, emit, mid_barrier); break;
     default: break;
   }
@@ -365,7 +402,9 @@ __device__ __forceinline__ void filter_dispatch(int L, const FftStage& sg, const
     case 2: if constexpr (E % 2 == 0) stage_filter<C, E, 2>(L, sg, tw, tid, nthr, load, mul, emit, mid_barrier); break;
     case 3: if constexpr (E % 3 == 0) stage_filter<C, E, 3>(L, sg, tw, tid, nthr, load, mul, emit, mid_barrier); break;
     case 4: if constexpr (E % 4 == 0) stage_filter<C, E, 4>(L, sg, tw, tid, nthr, load, mul, emit, mid_barrier); break;
+    case 6: if constexpr (fused<C, E>) stage_filter<C, E, 6>(L, sg, tw, tid, nthr, load, mul, emit, mid_barrier); break;
     case 8: if constexpr (E % 8 == 0) stage_filter<C, E, 8>(L, sg, tw, tid, nthr, load, mul, emit, mid_barrier); break;
+    case 12: if constexpr (fused<C, E>) stage_filter<C, E, 12>(L, sg, tw, tid, nthr, load, mul, emit, mid_barrier); break;
     case 16: if constexpr (E % 16 == 0) stage_filter<C, E, 16>(L, sg, tw, tid, nthr, load, mul, emit, mid_barrier); break;
     default: break;
   }
@@ -448,11 +487,23 @@ struct CtPlan {
   __host__ __device__ static constexpr int ns(int q) { return q == 0 ? 1 : ns(q - 1) * rad(q - 1); }
 };
 
+// The same for a length with a factor 3: the fused radices of plan.h.
+template <int L, int E, bool REV>
+struct CtFused {
+  static constexpr RadixSeq seq = fused_radices(L, E);
+  static constexpr int n = seq.n;
+  __host__ __device__ static constexpr int rad(int q) { return seq.r[REV ? n - 1 - q : q]; }
+  __host__ __device__ static constexpr int ns(int q) { return q == 0 ? 1 : ns(q - 1) * rad(q - 1); }
+};
+template <int L, int E, bool REV, bool FUSED> struct CtOf { using P = CtPlan<L, E, REV>; };
+template <int L, int E, bool REV> struct CtOf<L, E, REV, true> { using P = CtFused<L, E, REV>; };
+template <int L, int E, bool REV> using Ct = typename CtOf<L, E, REV, L % 3 == 0>::P;
+
 // True when plan p is exactly CtPlan<L, E, REV> (length, stage count and
 // every radix); the fixed path runs only then.
 template <int L, int E, bool REV>
-__device__ __forceinline__ bool ct_matches(const FftPlan& p) {
-  using P = CtPlan<L, E, REV>;
+__host__ __device__ __forceinline__ bool ct_matches(const FftPlan& p) {
+  using P = Ct<L, E, REV>;
   if (p.L != L || p.nst != P::n) return false;
   bool ok = true;
   if constexpr (P::n > 0) ok = ok && p.st[0].radix == P::rad(0);
@@ -466,7 +517,7 @@ __device__ __forceinline__ bool ct_matches(const FftPlan& p) {
 template <typename C, int E, bool INV, int L, bool REV, int Q, class Load, class Emit>
 __device__ __forceinline__ void ct_stage(const FftPlan& p, const C* __restrict__ tw, int tid, int nthr, Load& load,
                                          Emit& emit, bool mid_barrier) {
-  using P = CtPlan<L, E, REV>;
+  using P = Ct<L, E, REV>;
   constexpr int R = P::rad(Q);
   if constexpr (E % R == 0)
     stage_io<C, E, R, INV, L / R, P::ns(Q)>(L, stage_at(p, Q), tw, tid, nthr, load, emit, mid_barrier);
@@ -476,7 +527,7 @@ __device__ __forceinline__ void ct_stage(const FftPlan& p, const C* __restrict__
 template <typename C, int E, bool INV, int L, class Load, class Emit>
 __device__ __forceinline__ void fft_run_ct(C* s, int ld, const FftPlan& p, int tid, int nthr, Load& load, Emit& emit,
                                            bool load_from_tile, bool emit_to_tile) {
-  using P = CtPlan<L, E, false>;
+  using P = Ct<L, E, false>;
   constexpr int n = P::n;
   const C* tw = reinterpret_cast<const C*>(p.tw);
   SmemRows<C> rows{s, ld};
@@ -514,7 +565,7 @@ __device__ __forceinline__ bool fft_run_fixed(C* s, int ld, const FftPlan& p, in
 template <typename C, int E, int L, class Load, class Mul, class Emit>
 __device__ __forceinline__ void fft_filter_run_ct(C* s, int ld, const FftPlan& fwd, const FftPlan& inv, int tid,
                                                   int nthr, Load& load, Mul& mul, Emit& emit) {
-  using P = CtPlan<L, E, false>;
+  using P = Ct<L, E, false>;
   constexpr int n = P::n;
   constexpr int RF = P::rad(n - 1);
   const C* tw = reinterpret_cast<const C*>(fwd.tw);

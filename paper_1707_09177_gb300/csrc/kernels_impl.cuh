@@ -1,5 +1,6 @@
 // Definition of the launchers for one precision; included by kernels_f32.cu
-// and kernels_f64.cu with GAD_REAL set to float or double.
+// and kernels_f64.cu with GAD_REAL set to float or double. The FFT pass kernels
+// of each (precision, E) are compiled in units of their own (kernels_e.cu).
 #pragma once
 
 #include <algorithm>
@@ -11,33 +12,6 @@
 #include "stats.cuh"
 
 namespace gad {
-
-// Dynamic shared memory above 48 KB per block needs an opt-in; the kernels'
-// static shared memory (reduction scratch, mbarrier: under 1 KB) counts
-// against the same limit, so the opt-in is made with this margin.
-constexpr size_t kStaticSmemMargin = 4096;
-
-template <typename T, int E>
-static cudaError_t launch_pass_e(int kind, dim3 grid, int threads, size_t smem, cudaStream_t s,
-                                 const PassArgs<T>& a) {
-  void (*fn)(PassArgs<T>) = nullptr;
-  switch (kind) {
-    case PK_XFWD: fn = k_xfwd<T, E>; break;
-    case PK_XINV: fn = k_xinv<T, E>; break;
-    case PK_FILT: fn = k_filt<T, E>; break;
-    case PK_YFWD: fn = k_yfwd<T, E>; break;
-    case PK_YINV: fn = k_yinv<T, E>; break;
-    case PK_LFWD: fn = k_lfwd<T, E>; break;
-    case PK_LINV: fn = k_linv<T, E>; break;
-    default: return cudaErrorInvalidValue;
-  }
-  if (smem + kStaticSmemMargin > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  fn<<<grid, threads, smem, s>>>(a);
-  return cudaGetLastError();
-}
 
 template <typename T>
 cudaError_t launch_pass(int kind, int E, dim3 grid, int threads, size_t smem, cudaStream_t s,
@@ -53,6 +27,8 @@ cudaError_t launch_pass(int kind, int E, dim3 grid, int threads, size_t smem, cu
   }
   if (E == 16) return launch_pass_e<T, 16>(kind, grid, threads, smem, s, a);
   if (E == 24) return launch_pass_e<T, 24>(kind, grid, threads, smem, s, a);
+  if (E == 4) return launch_pass_e<T, 4>(kind, grid, threads, smem, s, a);
+  if (E == 12) return launch_pass_e<T, 12>(kind, grid, threads, smem, s, a);
   return cudaErrorInvalidValue;
 }
 

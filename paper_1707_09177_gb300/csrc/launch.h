@@ -16,11 +16,26 @@ enum PassKind : int {
   PK_STEN = 8,   // preconditioner z = M r with the dot (r, z), W rows per block (stencil.cuh)
 };
 
-// Launches pass `kind` with per-thread element count E (16 or 24). Returns the
+// Launches pass `kind` with per-thread element count E (4, 12, 16 or 24). Returns the
 // launch error (cudaSuccess when enqueued).
 template <typename T>
 cudaError_t launch_pass(int kind, int E, dim3 grid, int threads, size_t smem, cudaStream_t s,
                         const PassArgs<T>& a);
+
+// The same for one E (kernels_e.cu, one translation unit per precision and E).
+template <typename T, int E>
+cudaError_t launch_pass_e(int kind, dim3 grid, int threads, size_t smem, cudaStream_t s, const PassArgs<T>& a);
+
+// The float32 pass kernel of 12 elements per thread compiled for the plan's own
+// length (kernels_fused.cu), or nullptr when there is none.
+using PassKernelF = void (*)(PassArgs<float>);
+PassKernelF fused_kernel(int kind, const PassArgs<float>& a);
+PassKernelF fused_kernel_long(int kind, const PassArgs<float>& a);
+
+// Dynamic shared memory above 48 KB per block needs an opt-in; the kernels'
+// static shared memory (reduction scratch, mbarrier: under 1 KB) counts
+// against the same limit, so the opt-in is made with this margin.
+constexpr size_t kStaticSmemMargin = 4096;
 
 // One pass kind over several shape groups (k_multi): `args` (device) holds
 // each group's PassArgs (vgx, vgy its own launch shape), `start` (device,
@@ -28,6 +43,10 @@ cudaError_t launch_pass(int kind, int E, dim3 grid, int threads, size_t smem, cu
 template <typename T>
 cudaError_t launch_multi(int kind, int E, int blocks, int threads, size_t smem, cudaStream_t s,
                          const PassArgs<T>* args, const int* start, int ngroups);
+
+template <typename T, int E>
+cudaError_t launch_multi_e(int kind, int blocks, int threads, size_t smem, cudaStream_t s, const PassArgs<T>* args,
+                           const int* start, int ngroups);
 
 // Ends a deferred dot pass of `nblk` blocks per field and `batch` fields.
 template <typename T>

@@ -109,18 +109,19 @@ struct StaticPass {
 
 // The same plan and tile shape as the context-owning entry points build
 // (plan.h), so the pass kernels take the same code paths.
-bool plan_s(int L, int slots, int div, size_t cs, const void* tab, const void* tab_inv, StaticPass& pc) {
-  const int E = pick_E(L);
+bool plan_s(int L, int slots, int div, long long nseq, bool transposed, size_t cs, const void* tab,
+            const void* tab_inv, StaticPass& pc) {
+  if (!choose_pass(L, slots, div, nseq, transposed, cs, pc.t)) return false;
+  const int E = plan_E(L, pc.t.E, cs);
   if (!make_fft(L, E, tab, pc.fft)) return false;
-  if (tab_inv && !make_fft(L, E, tab_inv, pc.fft_inv, true)) return false;
-  return choose_tile(L, E, slots, div, cs, pc.t);
+  return !tab_inv || make_fft(L, E, tab_inv, pc.fft_inv, true);
 }
 
 // Fills a plan's twiddle table on the device (stream order).
 template <typename C, typename R>
-bool plan_table_s(int L, bool reversed, C* tw, cudaStream_t st) {
+bool plan_table_s(int L, int E, bool reversed, C* tw, cudaStream_t st) {
   RadixList rl{};
-  rl.n = plan_radices(L, pick_E(L), reversed, rl.r);
+  rl.n = plan_radices(L, E, reversed, rl.r);
   if (rl.n == 0) return false;
   if (L > 1) k_static_plan_twiddles<C, R><<<(L - 1 + 255) / 256, 256, 0, st>>>(tw, rl, L);
   return true;
@@ -158,9 +159,9 @@ ad_status run_static(const ad_grid* g, const void* in, void* out, int batch, cud
 
   StaticPass xf, fl, yf;
   const int nseq = g->ndim == 3 ? kxn * ny : kxn;
-  bool ok = plan_s(M, M + 1, pow2_part(ny), cs, tpx_d, nullptr, xf);
-  ok = ok && plan_s(Lf, Lf, 0, cs, tpf_d, tpfi_d, fl);
-  if (g->ndim == 3) ok = ok && plan_s(ny, ny, pow2_part(nz), cs, tpy_d, nullptr, yf);
+  bool ok = plan_s(M, M + 1, pow2_part(ny), (long long)ny * nz, true, cs, tpx_d, nullptr, xf);
+  ok = ok && plan_s(Lf, Lf, 0, nseq, false, cs, tpf_d, tpfi_d, fl);
+  if (g->ndim == 3) ok = ok && plan_s(ny, ny, pow2_part(nz), (long long)kxn * nz, true, cs, tpy_d, nullptr, yf);
   if (!ok) return AD_ERR_ARG;
   xf.rcp_a = 1.0f / (float)(nx / 4);
   xf.rcp_b = 1.0f / (float)(M / 2 + 1);
@@ -169,8 +170,9 @@ ad_status run_static(const ad_grid* g, const void* in, void* out, int batch, cud
   if (g->ndim == 3) yf.grid = dim3(kxn * (nz / yf.t.W), batch);
 
   k_static_twiddles<C, T><<<(nx + 255) / 256, 256, 0, st>>>(twx, nx);
-  ok = plan_table_s<C, T>(M, false, tpx_d, st) && plan_table_s<C, T>(Lf, false, tpf_d, st) &&
-       plan_table_s<C, T>(Lf, true, tpfi_d, st) && (g->ndim != 3 || plan_table_s<C, T>(ny, false, tpy_d, st));
+  ok = plan_table_s<C, T>(M, plan_E(M, xf.t.E, cs), false, tpx_d, st) && plan_table_s<C, T>(Lf, plan_E(Lf, fl.t.E, cs), false, tpf_d, st) &&
+       plan_table_s<C, T>(Lf, plan_E(Lf, fl.t.E, cs), true, tpfi_d, st) &&
+       (g->ndim != 3 || plan_table_s<C, T>(ny, plan_E(ny, yf.t.E, cs), false, tpy_d, st));
   if (!ok) return AD_ERR_ARG;
   if (cudaGetLastError() != cudaSuccess) return AD_ERR_CUDA;
 

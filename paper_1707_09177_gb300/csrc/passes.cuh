@@ -429,18 +429,38 @@ __device__ __forceinline__ void block_finish(const PassArgs<T>& a, const Acc<T>*
 // at once without holding registers. Ends with the copies complete and a
 // barrier.
 template <typename C>
+__device__ __forceinline__ void cp_async_elem(C* dst, const C* src) {
+  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+  if constexpr (sizeof(C) == 8)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
+
+// Visits the elements (w, i) of a W x n tile in the order of the transposed
+// global layout: move(shared pointer, global pointer). Where at least 16 threads
+// share a row a thread keeps it and its pointers advance by constants.
+template <typename C, typename G, class Move>
+__device__ __forceinline__ void walk_transposed(C* s, int ld, G* g, long long gstride, int W, int n, int tid, int nthr,
+                                                Move move) {
+  const int lw = __ffs(W) - 1;
+  if ((nthr & (16 * W - 1)) == 0) {
+    const int k0 = tid >> lw, dk = nthr >> lw;
+    C* row = s + (tid & (W - 1)) * ld;
+    G* gp = g + (tid & (W - 1)) + (long long)k0 * gstride;
+    const long long dg = dk * gstride;
+#pragma unroll 4
+    for (int k = k0; k < n; k += dk, gp += dg) move(row + phys(k), gp);
+  } else {
+    for (int idx = tid; idx < W * n; idx += nthr)
+      move(s + (idx & (W - 1)) * ld + phys(idx >> lw), g + (long long)(idx >> lw) * gstride + (idx & (W - 1)));
+  }
+}
+
+template <typename C>
 __device__ __forceinline__ void load_transposed(C* s, int ld, const C* __restrict__ g, long long gstride, int W,
                                                 int n, int tid, int nthr) {
-  const int lw = __ffs(W) - 1;
-  const int total = W * n;
-  for (int idx = tid; idx < total; idx += nthr) {
-    const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(s + (idx & (W - 1)) * ld + phys(idx >> lw)));
-    const C* src = g + (long long)(idx >> lw) * gstride + (idx & (W - 1));
-    if constexpr (sizeof(C) == 8)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
-    else
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-  }
+  walk_transposed(s, ld, g, gstride, W, n, tid, nthr, [](C* sp, const C* gp) { cp_async_elem(sp, gp); });
   asm volatile("cp.async.commit_group;\n" ::: "memory");
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   __syncthreads();
@@ -448,11 +468,28 @@ __device__ __forceinline__ void load_transposed(C* s, int ld, const C* __restric
 
 // Stores the shared-memory rows transposed (element (w, i) to g[i*gstride + w]).
 template <typename C>
-__device__ __forceinline__ void store_transposed(const C* s, int ld, C* __restrict__ g, long long gstride, int W,
+__device__ __forceinline__ void store_transposed(C* s, int ld, C* __restrict__ g, long long gstride, int W,
                                                  int n, int tid, int nthr) {
-  const int lw = __ffs(W) - 1;
-  for (int idx = tid; idx < W * n; idx += nthr)
-    g[(long long)(idx >> lw) * gstride + (idx & (W - 1))] = s[(idx & (W - 1)) * ld + phys(idx >> lw)];
+  walk_transposed(s, ld, g, gstride, W, n, tid, nthr, [](C* sp, C* gp) { *gp = *sp; });
+}
+
+// Visits the pairs (k, M - k), k = 0 .. M/2, of every row of a tile (the real
+// split and its inverse): visit(row, k). A thread keeps its row where a whole
+// warp or more works on one (fewer threads per row would scatter a warp over
+// several rows' banks).
+template <typename C, class Visit>
+__device__ __forceinline__ void walk_pairs(C* s, int ld, int W, int M, float rcp_h1, int tid, int nthr, Visit visit) {
+  const int h1 = (M >> 1) + 1;
+  if ((nthr & (32 * W - 1)) == 0) {
+    const int tpr = nthr >> (__ffs(W) - 1), w = tid / tpr;
+    C* row = s + w * ld;
+    for (int k = tid - w * tpr; k < h1; k += tpr) visit(row, k);
+  } else {
+    for (int idx = tid; idx < W * h1; idx += nthr) {
+      const int w = fquot(idx, rcp_h1);
+      visit(s + w * ld, idx - w * h1);
+    }
+  }
 }
 
 template <typename T> struct V2 { T x, y; };
@@ -471,10 +508,10 @@ template <typename T> __device__ __forceinline__ void st2(T* p, T a, T b) {
 // a few spilled words cost less than the latency the extra warps hide
 // (measured: the filter pass 28-31% faster than at 2 blocks and 128
 // registers, the x/y passes 5-17% faster than at 3 blocks and 80). Float32,
-// E = 24 (radix-3 lengths): 3 blocks per SM (14-15% faster per pass than 2 at
+// E = 24 (long radix-3 lengths): 3 blocks per SM (14-15% faster per pass than 2 at
 // 384^3 and 1536^2). Float64: 2 blocks.
-#define GAD_BOUNDS(T, E) __launch_bounds__(256, sizeof(T) == 4 ? ((E) == 16 ? 4 : 3) : 2)
-#define GAD_BOUNDS_FILT(T, E) __launch_bounds__(256, sizeof(T) == 4 ? ((E) == 16 ? 4 : 3) : 2)
+#define GAD_BOUNDS(T, E) __launch_bounds__(256, sizeof(T) == 4 ? ((E) == 24 ? 3 : 4) : 2)
+#define GAD_BOUNDS_FILT(T, E) __launch_bounds__(256, sizeof(T) == 4 ? ((E) == 24 ? 3 : 4) : 2)
 
 // ---------------------------------------------------------------------------
 // Row-tile streaming for the fused Krylov prologue/epilogue of the x passes.
@@ -507,18 +544,15 @@ __device__ __forceinline__ void stream_tile(int W, int nx, float rcp_q, long lon
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int c = c0 + u * nthr;
-      if (c < total) {
-        const int w = fquot(c, rcp_q);
-        ld(u, base + (long long)w * nx + 4 * (c - w * qn));
-      }
+      if (c < total) ld(u, base + 4 * c);
+
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int c = c0 + u * nthr;
       if (c < total) {
         const int w = fquot(c, rcp_q);
-        const int q = c - w * qn;
-        fin(u, w, q, base + (long long)w * nx + 4 * q);
+        fin(u, w, c - w * qn, base + 4 * c);
       }
     }
   }
@@ -777,7 +811,7 @@ __device__ __forceinline__ void xinv_epilogue(const PassArgs<T>& a, const typena
 // half-length FFT runs in shared memory, followed by the real-to-complex
 // split and the transposed store to S1.
 //   rcp_a = 1/(nx/4), rcp_b = 1/(nx/4 + 1)
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __device__ __forceinline__ void xfwd_body(const PassArgs<T>& a, const VBlock& vb) {
   using C = typename cpx<T>::t;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -814,44 +848,43 @@ __device__ __forceinline__ void xfwd_body(const PassArgs<T>& a, const VBlock& vb
   xfwd_prologue<T, 2>(a, s, base, first, al, be, om, tid, nthr, f);
   __syncthreads();
   SmemRows<C> rows{s, a.ld};
-  if (!fft_run_fixed<C, E, false, 1024>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true) &&
+  if constexpr (LC > 0)
+    fft_run_ct<C, E, false, LC>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true);
+  else if (!fft_run_fixed<C, E, false, 1024>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true) &&
       !fft_run_fixed<C, E, false, 256>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true) &&
       !fft_run_fixed<C, E, false, 128>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true))
     fft_run<C, E, false>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true);
   // split the packed half-length transform into the real-input spectrum
   const C* twx = reinterpret_cast<const C*>(a.twx);
-  const int h1 = (M >> 1) + 1;
-  for (int idx = tid; idx < a.W * h1; idx += nthr) {
-    const int w = fquot(idx, a.rcp_b);
-    const int k = idx - w * h1;
-    C* row = s + w * a.ld;
+  walk_pairs(s, a.ld, a.W, M, a.rcp_b, tid, nthr, [&](C* row, int k) {
     if (k == 0) {
       const C z0 = row[0];
       row[0] = C{z0.x + z0.y, T(0)};
       row[phys(M)] = C{z0.x - z0.y, T(0)};
     } else {
-      const C A = row[phys(k)], B = row[phys(M - k)];
+      C &ra = row[phys(k)], &rb = row[phys(M - k)];
+      const C A = ra, B = rb;
       const C e = {T(0.5) * (A.x + B.x), T(0.5) * (A.y - B.y)};   // (A + conj B)/2
       const C o = {T(0.5) * (A.y + B.y), T(0.5) * (B.x - A.x)};   // -i (A - conj B)/2
       const C wo = cmul(twx[k], o);
-      row[phys(k)] = cadd(e, wo);
-      row[phys(M - k)] = cconj(csub(e, wo));
+      ra = cadd(e, wo);
+      rb = cconj(csub(e, wo));
     }
-  }
+  });
   __syncthreads();
   C* S1 = reinterpret_cast<C*>(a.S1) + (long long)f * a.SP + (long long)z * a.kxn * a.ny + y0;
   store_transposed(s, a.ld, S1, a.ny, a.W, M + 1, tid, nthr);
 }
 
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __global__ void GAD_BOUNDS(T, E) k_xfwd(const __grid_constant__ PassArgs<T> a) {
-  xfwd_body<T, E>(a, own_block());
+  xfwd_body<T, E, LC>(a, own_block());
 }
 
 // Inverse x pass: transposed load from S1, complex-to-real preparation, FFT
 // in shared memory, then the fused epilogue and dots streamed over the row
 // tile.
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __device__ __forceinline__ void xinv_body(const PassArgs<T>& a, const VBlock& vb) {
   using C = typename cpx<T>::t;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -870,26 +903,25 @@ __device__ __forceinline__ void xinv_body(const PassArgs<T>& a, const VBlock& vb
     const C* S1 = reinterpret_cast<const C*>(a.S1) + (long long)f * a.SP + (long long)z * a.kxn * a.ny + y0;
     load_transposed(s, a.ld, S1, a.ny, a.W, M + 1, tid, nthr);
     const C* twx = reinterpret_cast<const C*>(a.twx);
-    const int h1 = (M >> 1) + 1;
-    for (int idx = tid; idx < a.W * h1; idx += nthr) {
-      const int w = fquot(idx, a.rcp_b);
-      const int k = idx - w * h1;
-      C* row = s + w * a.ld;
+    walk_pairs(s, a.ld, a.W, M, a.rcp_b, tid, nthr, [&](C* row, int k) {
       if (k == 0) {
         const T x0 = row[0].x, xm = row[phys(M)].x;   // imaginary parts of DC/Nyquist dropped
         row[0] = C{x0 + xm, x0 - xm};
       } else {
-        const C A = row[phys(k)], B = row[phys(M - k)];
+        C &ra = row[phys(k)], &rb = row[phys(M - k)];
+        const C A = ra, B = rb;
         const C e = {A.x + B.x, A.y - B.y};            // A + conj B
         const C d = {A.x - B.x, A.y + B.y};            // A - conj B
         const C o = cmulc(d, twx[k]);                  // (A - conj B) conj(W^k)
-        row[phys(k)] = C{e.x - o.y, e.y + o.x};        // e + i o
-        row[phys(M - k)] = C{e.x + o.y, o.x - e.y};    // conj(e) + i conj(o)
+        ra = C{e.x - o.y, e.y + o.x};                  // e + i o
+        rb = C{e.x + o.y, o.x - e.y};                  // conj(e) + i conj(o)
       }
-    }
+    });
     __syncthreads();
     SmemRows<C> rows{s, a.ld};
-    if (!fft_run_fixed<C, E, true, 1024>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true) &&
+    if constexpr (LC > 0)
+      fft_run_ct<C, E, true, LC>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true);
+    else if (!fft_run_fixed<C, E, true, 1024>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true) &&
         !fft_run_fixed<C, E, true, 256>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true) &&
         !fft_run_fixed<C, E, true, 128>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true))
       fft_run<C, E, true>(s, a.ld, a.fft, tid, a.tfft, rows, rows, true, true);
@@ -925,9 +957,9 @@ __device__ __forceinline__ void xinv_body(const PassArgs<T>& a, const VBlock& vb
   if (a.ndots) block_finish(a, acc, f, act, vb);
 }
 
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __global__ void GAD_BOUNDS(T, E) k_xinv(const __grid_constant__ PassArgs<T> a) {
-  xinv_body<T, E>(a, own_block());
+  xinv_body<T, E, LC>(a, own_block());
 }
 
 // Filter pass along the last axis (y in 2D, z in 3D): forward FFT of W
@@ -935,7 +967,7 @@ __global__ void GAD_BOUNDS(T, E) k_xinv(const __grid_constant__ PassArgs<T> a) {
 // G_hat(k)/P with Parseval dots in registers, inverse FFT written straight
 // back. fft holds the forward plan, fft_inv the reversed one. In 3D the
 // sequence index is kx*ny + ky.
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __device__ __forceinline__ void filt_body(const PassArgs<T>& a, const VBlock& vb) {
   using C = typename cpx<T>::t;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1003,7 +1035,9 @@ __device__ __forceinline__ void filt_body(const PassArgs<T>& a, const VBlock& vb
     auto emit = [&](int w, int i, const C& x) {
       if (w < nvalid) S[(long long)w * L + i] = x;
     };
-    if (!fft_filter_run_fixed<C, E, 2048>(s, a.ld, a.fft, a.fft_inv, tid, a.tfft, load, mul, emit) &&
+    if constexpr (LC > 0)
+      fft_filter_run_ct<C, E, LC>(s, a.ld, a.fft, a.fft_inv, tid, a.tfft, load, mul, emit);
+    else if (!fft_filter_run_fixed<C, E, 2048>(s, a.ld, a.fft, a.fft_inv, tid, a.tfft, load, mul, emit) &&
         !fft_filter_run_fixed<C, E, 512>(s, a.ld, a.fft, a.fft_inv, tid, a.tfft, load, mul, emit) &&
         !fft_filter_run_fixed<C, E, 256>(s, a.ld, a.fft, a.fft_inv, tid, a.tfft, load, mul, emit))
       fft_filter_run<C, E>(s, a.ld, a.fft, a.fft_inv, tid, a.tfft, load, mul, emit);
@@ -1014,15 +1048,15 @@ __device__ __forceinline__ void filt_body(const PassArgs<T>& a, const VBlock& vb
   if (a.ndots) block_finish(a, acc, f, act, vb);
 }
 
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __global__ void GAD_BOUNDS_FILT(T, E) k_filt(const __grid_constant__ PassArgs<T> a) {
-  filt_body<T, E>(a, own_block());
+  filt_body<T, E, LC>(a, own_block());
 }
 
 // 3D forward y pass: W consecutive z at one kx; the first stage reads the
 // S1 rows [z][kx][:] directly, the tile is stored transposed into S2
 // [kx][ky][z].  Grid x = kxn * (nz/W).
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __device__ __forceinline__ void yfwd_body(const PassArgs<T>& a, const VBlock& vb) {
   using C = typename cpx<T>::t;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1037,21 +1071,23 @@ __device__ __forceinline__ void yfwd_body(const PassArgs<T>& a, const VBlock& vb
   const int kxn = a.kxn;
   auto load = [&](int w, int i) -> C { return S1[((long long)(z0 + w) * kxn + kx) * L + i]; };
   SmemRows<C> rows{s, a.ld};
-  if (!fft_run_fixed<C, E, false, 512>(s, a.ld, a.fft, tid, a.tfft, load, rows, false, true) &&
+  if constexpr (LC > 0)
+    fft_run_ct<C, E, false, LC>(s, a.ld, a.fft, tid, a.tfft, load, rows, false, true);
+  else if (!fft_run_fixed<C, E, false, 512>(s, a.ld, a.fft, tid, a.tfft, load, rows, false, true) &&
       !fft_run_fixed<C, E, false, 256>(s, a.ld, a.fft, tid, a.tfft, load, rows, false, true))
     fft_run<C, E, false>(s, a.ld, a.fft, tid, a.tfft, load, rows, false, true);
   C* S2 = reinterpret_cast<C*>(a.S2) + (long long)f * a.SP + (long long)kx * L * a.nz + z0;
   store_transposed(s, a.ld, S2, a.nz, a.W, L, tid, nthr);
 }
 
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __global__ void GAD_BOUNDS(T, E) k_yfwd(const __grid_constant__ PassArgs<T> a) {
-  yfwd_body<T, E>(a, own_block());
+  yfwd_body<T, E, LC>(a, own_block());
 }
 
 // 3D inverse y pass: transposed load from S2, inverse FFT whose last stage
 // writes the S1 rows directly.
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __device__ __forceinline__ void yinv_body(const PassArgs<T>& a, const VBlock& vb) {
   using C = typename cpx<T>::t;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1068,14 +1104,16 @@ __device__ __forceinline__ void yinv_body(const PassArgs<T>& a, const VBlock& vb
   const int kxn = a.kxn;
   auto emit = [&](int w, int i, const C& x) { S1[((long long)(z0 + w) * kxn + kx) * L + i] = x; };
   SmemRows<C> rows{s, a.ld};
-  if (!fft_run_fixed<C, E, true, 512>(s, a.ld, a.fft, tid, a.tfft, rows, emit, true, false) &&
+  if constexpr (LC > 0)
+    fft_run_ct<C, E, true, LC>(s, a.ld, a.fft, tid, a.tfft, rows, emit, true, false);
+  else if (!fft_run_fixed<C, E, true, 512>(s, a.ld, a.fft, tid, a.tfft, rows, emit, true, false) &&
       !fft_run_fixed<C, E, true, 256>(s, a.ld, a.fft, tid, a.tfft, rows, emit, true, false))
     fft_run<C, E, true>(s, a.ld, a.fft, tid, a.tfft, rows, emit, true, false);
 }
 
-template <typename T, int E>
+template <typename T, int E, int LC = 0>
 __global__ void GAD_BOUNDS(T, E) k_yinv(const __grid_constant__ PassArgs<T> a) {
-  yinv_body<T, E>(a, own_block());
+  yinv_body<T, E, LC>(a, own_block());
 }
 
 // One pass over several shape groups in a single launch: block b belongs to

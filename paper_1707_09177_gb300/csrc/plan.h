@@ -36,9 +36,13 @@ inline int pick_E(int L) { return (L % 3 == 0) ? 24 : 16; }
 
 constexpr int kMaxStages = 5;       // the kernels unroll at most 5 stages
 
+// Elements per FFT thread on a grid too small to fill the GPU (choose_pass):
+// four to six times as many threads, each with a shorter chain.
+inline int small_E(int L) { return (L % 3 == 0) ? 12 : 4; }
+
 // Balanced radix list for a length L and E elements per thread: the factors 3
 // first, then the power of two split into as few stages of at most 2^4 (E =
-// 16) or 2^3 (E = 24) as possible, the larger radices first. Writes at most
+// 16), 2^3 (E = 24) or 2^2 (E = 4, 12) as possible, the larger radices first. Writes at most
 // kMaxStages radices into rad and returns their number, or 0 when L is not
 // 2^a 3^b, a radix does not divide E, or more stages would be needed.
 inline int radices_for(int L, int E, int* rad) {
@@ -47,7 +51,7 @@ inline int radices_for(int L, int E, int* rad) {
   while (n > 1 && n % 3 == 0) { n /= 3; ++b; }
   if (n != 1 || (a == 0 && b == 0)) return 0;
   if (b > 0 && E % 3 != 0) return 0;
-  const int maxlog = (E % 16 == 0) ? 4 : 3;
+  const int maxlog = (E % 16 == 0) ? 4 : (E % 8 == 0) ? 3 : 2;
   const int ns = a > 0 ? (a + maxlog - 1) / maxlog : 0;
   if (b + ns > kMaxStages) return 0;
   int k = 0;
@@ -57,6 +61,52 @@ inline int radices_for(int L, int E, int* rad) {
     if (E % rad[i] != 0) return 0;
   return k;
 }
+
+// Radices of the float32 plans of lengths with a factor 3 (E = 12): the fewest
+// stages from 12, 6, 4, 3 and 2 (ties go to the smaller sum), so that a factor
+// 3 shares a stage with a power of two instead of taking one of its own (288:
+// 4 6 12 instead of 3 3 8 4). Powers of two
+// come first: the first stage writes with a stride of its radix, which is free
+// of bank conflicts for them. n = 0 when there is no such plan.
+struct RadixSeq {
+  int n = 0, sum = 0;
+  int r[kMaxStages] = {};
+};
+
+constexpr RadixSeq fused_search(int L, int E, int top, int depth) {
+  RadixSeq best{};
+  if (L == 1 || depth == kMaxStages) return best;
+  const int cand[5] = {12, 6, 4, 3, 2};
+  for (int i = 0; i < 5; ++i) {
+    const int c = cand[i];
+    if (c > top || E % c != 0 || L % c != 0) continue;
+    RadixSeq s = fused_search(L / c, E, c, depth + 1);
+    if (L / c != 1 && s.n == 0) continue;
+    s.r[s.n] = c;
+    s.n += 1;
+    s.sum += c;
+    if (best.n == 0 || s.n < best.n || (s.n == best.n && s.sum < best.sum)) best = s;
+  }
+  return best;
+}
+
+constexpr RadixSeq fused_radices(int L, int E) {
+  RadixSeq s = fused_search(L, E, 12, 0), o{};
+  for (int pow2 = 1; pow2 >= 0; --pow2)
+    for (int i = 0; i < s.n; ++i)                 // s.r ascends
+      if ((s.r[i] % 3 != 0) == (pow2 != 0)) o.r[o.n++] = s.r[i];
+  return o;
+}
+
+// Lengths of those plans, at 12 elements per thread: 64 registers and 4 blocks
+// per SM with nothing spilled (the filter pass at 24 elements spills 900 bytes
+// per thread at 80 registers). A transposed tile of more than 768 elements per
+// row would hold fewer than the four rows of a 32-byte sector in 256 threads
+// and keeps 24 elements.
+constexpr bool fused_length(int L) { return L % 3 == 0 && L >= 36 && L <= 2304 && fused_radices(L, 12).n > 0; }
+
+// Key of a plan: its element count, odd for the fused radices.
+inline int plan_E(int L, int E, size_t csize) { return csize == 8 && E == 12 && fused_length(L) ? 13 : E; }
 
 // Stockham stage table for the radices rad[0..nrad) (in that order) over the
 // plan's twiddle table `tab` (see FftPlan; fill it with plan_twiddles).
@@ -85,7 +135,14 @@ inline bool make_fft_from(int L, const int* rad, int nrad, const void* tab, FftP
 // stage meets the forward transform's last stage in registers). Returns the
 // number of stages, 0 when there is no plan.
 inline int plan_radices(int L, int E, bool reversed, int* rad) {
-  const int n = radices_for(L, E, rad);
+  int n;
+  if (E & 1) {
+    const RadixSeq s = fused_radices(L, E - 1);
+    n = s.n;
+    for (int i = 0; i < n; ++i) rad[i] = s.r[i];
+  } else {
+    n = radices_for(L, E, rad);
+  }
   if (reversed)
     for (int i = 0; i < n / 2; ++i) {
       const int t = rad[i];
@@ -171,6 +228,74 @@ inline bool choose_tile(int L, int E, int slots, int div, size_t csize, TileShap
   ts.ld = ld;
   ts.smem = (size_t)bestW * ld * csize;
   return true;
+}
+
+// Blocks per field below which a pass cannot fill the GPU with the default
+// tile, and complex elements per field below which even 16 elements per
+// thread leave most of the 152 SMs' warp slots empty.
+constexpr int kWantBlocks = 152;
+constexpr long long kSmallElems = 152 * 64 * 16;
+
+// Row stride of a tile of W rows that is stored or loaded transposed (the W
+// values of one wavenumber by consecutive threads): the 128 bytes that a
+// shared-memory phase moves are then W rows of 128/csize/W consecutive
+// elements, which fall into distinct banks when the stride is that count
+// modulo 128/csize (an odd stride when a phase holds one element per row).
+// With the odd stride of tile_ld, W = 4 rows of float2 met in 7 of 16 bank pairs.
+inline int transposed_ld(int ld, int W, size_t csize) {
+  const int B = (int)(128 / csize);
+  if (W >= B || W < 2) return ld;
+  while (ld % B != B / W) ++ld;
+  return ld;
+}
+
+// Elements per thread and tile of a pass over `nseq` sequences of length L
+// per field. Default: 12 (fused_length) or pick_E(L) and choose_tile's 256-thread blocks, for
+// every grid that gives kWantBlocks of them. Smaller grids get narrower
+// tiles, the widest that still gives kWantBlocks, down to rows of 32 bytes
+// (one sector) in the transposed spectra and to one warp; grids under
+// kSmallElems also get small_E(L). The rule looks at one field, never at the
+// batch: the tile fixes the order of the dot sums, and a field's result must
+// not depend on the batch it is solved in.
+inline bool choose_pass(int L, int slots, int div, long long nseq, bool transposed, size_t csize, TileShape& ts,
+                        int want_T = 256) {
+  const int E0 = csize == 8 && fused_length(L) && !(transposed && L > 768) ? 12 : pick_E(L);
+  if (!choose_tile(L, E0, slots, div, csize, ts)) return false;
+  auto done = [&]() {
+    if (transposed) {
+      ts.ld = transposed_ld(ts.ld, ts.W, csize);
+      ts.smem = (size_t)ts.W * ts.ld * csize;
+    }
+    return true;
+  };
+  // the default tile narrowed to about `want_T` threads, rows of 32 bytes at least
+  while (ts.T > want_T && ts.W > 1 && (!transposed || ts.W * csize > 32)) {
+    ts.W /= 2;
+    ts.T /= 2;
+    ts.smem /= 2;
+  }
+  if ((nseq + ts.W - 1) / ts.W >= kWantBlocks) return done();
+  int rad[kMaxStages];
+  int E = E0;
+  if (nseq * L < kSmallElems && radices_for(L, small_E(L), rad) > 0) E = small_E(L);
+  TileShape best;
+  for (int W = 4096; W >= 1; W /= 2) {
+    if (div > 0 && div % W != 0) continue;
+    const long long tot = (long long)W * L;
+    if (tot % E != 0 || tot / E > 256) continue;
+    const size_t smem = (size_t)W * ts.ld * csize;
+    if (smem > 100 * 1024) continue;
+    const bool narrow = tot / E < 32 || (transposed && W * csize < 32);
+    if (best.W && narrow) break;
+    best.E = E;
+    best.W = W;
+    best.T = (int)(tot / E);
+    best.ld = ts.ld;
+    best.smem = smem;
+    if ((nseq + W - 1) / W >= kWantBlocks) break;
+  }
+  if (best.W) ts = best;
+  return done();
 }
 
 }  // namespace gad
