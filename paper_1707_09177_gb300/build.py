@@ -26,6 +26,7 @@ SOURCES = ([("kernels_e.cu", ("GAD_REAL=float", "GAD_E=16")), ("kernels_multi.cu
               if (t, e) != ("float", 16)]
            + [("kernels_multi.cu", ("GAD_E=%d" % e,)) for e in (24, 12, 4)]
            + [("kernels_fused.cu", ("GAD_LONG=%d" % g,)) for g in (1, 0)]
+           + [("kernels_cluster.cu", ("GAD_REAL=%s" % t,)) for t in ("float", "double")]
            + [(f, ()) for f in ("api.cu", "kernels_f32.cu", "kernels_f64.cu", "noalloc.cu", "cnn.cu", "conv_tc.cu")])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -49,6 +49,8 @@ struct Plan {
   long long P = 0, SP = 0;
   PassCfg xf, xi, fl, yf, yi;
   PassCfg sn;                        // preconditioner stencil pass (W rows per block)
+  ClusterShape cl;                   // csize > 0: small grid, solved by one cluster per field (cluster.cuh)
+  FftPlan clx{}, cll{};              // its plans
   const void* twx = nullptr;
   void *S1 = nullptr, *S2 = nullptr;
   void *R = nullptr, *Pv = nullptr, *Q = nullptr, *Sv = nullptr, *F0 = nullptr;
@@ -84,6 +86,13 @@ struct LaunchRec {
   PassArgs<double> ad{};
 };
 
+// One application of G as the drivers describe it.
+struct Fwd { int op = XF_COPY; const void* A = nullptr; const void* B = nullptr; void* O1 = nullptr; void* O2 = nullptr; void* O3 = nullptr;
+             bool clear_cond = false; };
+struct Flt { int op = FI_NONE; int stage = SS_NONE; };
+struct Inv { int op = XI_STORE; const void* A = nullptr; const void* B = nullptr; const void* C = nullptr;
+             void* O1 = nullptr; void* O2 = nullptr; int ndots = 0; int stage = SS_NONE; bool set_cond = false; };
+
 struct BatchedGroup {
   Plan* p = nullptr;
   std::vector<int> fields;          // indices into the caller's field arrays
@@ -116,6 +125,7 @@ struct ad_ctx {
   bool autotune = false;                      // tune the tiles of every new plan of a batched solve
   bool batched_multi = false;                 // batched solves: one launch per pass stage over all groups
   std::vector<LaunchRec>* record = nullptr;   // when set, pass launches are recorded, not issued
+  std::vector<ClusterStep>* steps = nullptr;  // when set, applications of G are collected for a cluster solve
   std::map<std::string, BatchedEntry> bgraphs;
   std::vector<cudaStream_t> branches;         // capture streams of the batched graph's branches
   std::vector<cudaEvent_t> events;
@@ -381,6 +391,20 @@ ad_status get_plan(ad_ctx* ctx, const ad_grid* g, int batch, Plan** out) {
     p->sn.rcp_a = 1.0f / (float)(p->nx / 4);
     p->sn.grid = dim3((unsigned)(tiles * (nmarch / chunk)), batch);
   }
+  if (cluster_shape(p->nx, p->ny, p->nz, cs, p->cl) &&
+      (p->f64 ? cluster_fits<double>(p->cl.csize, p->cl.threads, p->cl.smem)
+              : cluster_fits<float>(p->cl.csize, p->cl.threads, p->cl.smem))) {
+    const void *tx8 = nullptr, *tl8 = nullptr;
+    if ((s = get_plan_table(ctx, M, kClusterE, false, p->f64, &tx8)) != AD_OK ||
+        (s = get_plan_table(ctx, Lf, kClusterE, false, p->f64, &tl8)) != AD_OK) {
+      delete p;
+      return s;
+    }
+    ok = make_fft(M, kClusterE, tx8, p->clx) && make_fft(Lf, kClusterE, tl8, p->cll);
+    if (!ok) { delete p; return fail(ctx, AD_ERR_ARG, "no tiling for this grid"); }
+  } else {
+    p->cl = ClusterShape{};
+  }
   const size_t vb = (size_t)p->P * batch * rs, sb = (size_t)p->SP * batch * cs;
   if ((s = dmalloc(ctx, p, &p->S1, sb)) != AD_OK ||
       (p->ndim == 3 && (s = dmalloc(ctx, p, &p->S2, sb)) != AD_OK)) { free_plan(p); return s; }
@@ -466,11 +490,6 @@ ad_status ensure_hist(ad_ctx* ctx, Plan* p, int maxit) {
 
 // ---------------------------------------------------------------------------
 // Enqueueing one application of G with the given fused prologue/epilogue.
-struct Fwd { int op = XF_COPY; const void* A = nullptr; const void* B = nullptr; void* O1 = nullptr; void* O2 = nullptr; void* O3 = nullptr;
-             bool clear_cond = false; };
-struct Flt { int op = FI_NONE; int stage = SS_NONE; };
-struct Inv { int op = XI_STORE; const void* A = nullptr; const void* B = nullptr; const void* C = nullptr;
-             void* O1 = nullptr; void* O2 = nullptr; int ndots = 0; int stage = SS_NONE; bool set_cond = false; };
 struct Common { FieldState* st = nullptr; SolveConfig cfg{}; cudaGraphConditionalHandle cond = 0; bool in_graph = false; int force = 0;
                 int ncomp = 0, npairs = 0, pair_code = 0; unsigned long long wait_ns = 1000000000ull; };
 
@@ -545,8 +564,44 @@ cudaError_t issue(ad_ctx* ctx, int kind, const PassCfg& pc, cudaStream_t s, cons
 }
 
 template <typename T>
+ClusterArgs<T> cluster_args(const Plan* p, const Common& c) {
+  ClusterArgs<T> ca{};
+  const ClusterShape& s = p->cl;
+  const int own = p->ny / s.csize;
+  ca.a = base_args<T>(p, c);
+  ca.a.rcp_a = p->xf.rcp_a;
+  ca.fx = p->clx; ca.fl = p->cll;
+  ca.csize = s.csize; ca.buf = s.buf; ca.ldx = s.ldx; ca.ldl = s.ldl; ca.kc = s.kc;
+  ca.rcp_kc = 1.0f / (float)s.kc;
+  ca.rcp_own = 1.0f / (float)own;
+  ca.rcp_l = 1.0f / (float)p->ny;
+  return ca;
+}
+
+ClusterStep cluster_step(const Fwd& fw, const Flt& fl, const Inv& iv) {
+  ClusterStep t{};
+  t.xf = fw.op; t.fA = fw.A; t.fB = fw.B; t.fO1 = fw.O1; t.fO2 = fw.O2; t.fO3 = fw.O3;
+  t.fi = fl.op; t.fstage = fl.stage;
+  t.xi = iv.op; t.iA = iv.A; t.iB = iv.B; t.iC = iv.C; t.iO1 = iv.O1; t.iO2 = iv.O2;
+  t.ndots = iv.ndots; t.istage = iv.stage;
+  return t;
+}
+
+template <typename T>
 ad_status enqueue_G(ad_ctx* ctx, Plan* p, cudaStream_t s, const Fwd& fw, const Flt& fl, const Inv& iv,
                     const Common& c, int* nl) {
+  if (ctx->steps) {
+    ctx->steps->push_back(cluster_step(fw, fl, iv));
+    return AD_OK;
+  }
+  if (p->cl.csize && !c.st) {           // plain filtering of a small grid
+    ClusterArgs<T> ca = cluster_args<T>(p, c);
+    ca.n_init = 1;
+    ca.step[0] = cluster_step(fw, fl, iv);
+    CK(launch_cluster<T>(ca, p->batch, p->cl.threads, p->cl.smem, s));
+    ++*nl;
+    return AD_OK;
+  }
   PassArgs<T> a = base_args<T>(p, c);
   // forward x pass
   set_pass(a, p->xf);
@@ -792,6 +847,16 @@ ad_status enqueue_body(ad_ctx* ctx, Plan* p, cudaStream_t s, const SolveIO& io, 
   }
 }
 
+// The true residual of the returned u, one more application of G.
+template <typename T>
+ad_status enqueue_true(ad_ctx* ctx, Plan* p, cudaStream_t s, const SolveIO& io, const Common& c, int* nl) {
+  Common cf = c;
+  cf.force = 1;
+  Fwd fw; fw.op = XF_COPY; fw.A = io.u;
+  Inv iv; iv.op = XI_RES; iv.A = io.ubar; iv.ndots = 1; iv.stage = SS_TRUE;
+  return enqueue_G<T>(ctx, p, s, fw, Flt{}, iv, cf, nl);
+}
+
 template <typename T>
 ad_status enqueue_finish(ad_ctx* ctx, Plan* p, cudaStream_t s, const SolveIO& io, const Common& c, int* nl) {
   if (io.spectral) {
@@ -801,13 +866,34 @@ ad_status enqueue_finish(ad_ctx* ctx, Plan* p, cudaStream_t s, const SolveIO& io
     CK(launch_cg_finish<T>((T*)io.u, (const T*)p->Pv, p->st, p->P, p->batch, s));
     ++*nl;
   }
-  if (io.want_true) {
-    Common cf = c;
-    cf.force = 1;
-    Fwd fw; fw.op = XF_COPY; fw.A = io.u;
-    Inv iv; iv.op = XI_RES; iv.A = io.ubar; iv.ndots = 1; iv.stage = SS_TRUE;
-    return enqueue_G<T>(ctx, p, s, fw, Flt{}, iv, cf, nl);
-  }
+  return io.want_true ? enqueue_true<T>(ctx, p, s, io, c, nl) : AD_OK;
+}
+
+// A solve that one cluster per field runs in one launch: small grids, the
+// physical-space methods without a preconditioner. The choice depends on the
+// grid and the method only, so a field's result is the same alone, in a batch
+// and in a batched call.
+bool solves_in_cluster(const Plan* p, bool spectral, bool precond) { return p->cl.csize && !spectral && !precond; }
+
+template <typename T>
+ad_status enqueue_cluster_solve(ad_ctx* ctx, Plan* p, cudaStream_t s, const SolveIO& io, const Common& c) {
+  // the applications of G that the pass-launching drivers would issue
+  std::vector<ClusterStep> steps;
+  ClusterArgs<T> ca = cluster_args<T>(p, c);
+  int nl = 0;
+  ctx->steps = &steps;
+  ad_status st = enqueue_init_passes<T>(ctx, p, s, io, c, &nl);
+  ca.n_init = (int)steps.size();
+  if (st == AD_OK) st = enqueue_body<T>(ctx, p, s, io, c, &nl);
+  ca.n_body = (int)steps.size() - ca.n_init;
+  if (st == AD_OK && io.want_true) st = enqueue_true<T>(ctx, p, s, io, c, &nl);
+  ca.n_true = (int)steps.size() - ca.n_init - ca.n_body;
+  ctx->steps = nullptr;
+  if (st != AD_OK) return st;
+  if (steps.size() > sizeof ca.step / sizeof ca.step[0]) return fail(ctx, AD_ERR_ARG, "cluster solve steps");
+  for (size_t i = 0; i < steps.size(); ++i) ca.step[i] = steps[i];
+  if (io.method == AD_CG) { ca.cg_u = io.u; ca.cg_p = p->Pv; }
+  CK(launch_cluster<T>(ca, p->batch, p->cl.threads, p->cl.smem, s));
   return AD_OK;
 }
 
@@ -886,6 +972,12 @@ ad_status run_solve(ad_ctx* ctx, Plan* p, const SolveIO& io, double tol, int max
   c.cfg.hist = p->hist;
   c.cfg.hist_ld = p->hist_cap;
   ad_status st;
+  if (solves_in_cluster(p, io.spectral, io.precond)) {
+    if ((st = enqueue_cluster_solve<T>(ctx, p, stream, io, c)) != AD_OK) return st;
+    *loops_out = 0;
+    ctx->launches = 1;
+    return AD_OK;
+  }
   if (ctx->use_graph) {
     char buf[256];
     snprintf(buf, sizeof buf, "|%d|%d|%d|%a|%d|%p|%p|%p|%d", io.method, io.spectral ? 1 : 0, io.precond ? 1 : 0,
@@ -1223,7 +1315,20 @@ ad_status capture_group(ad_ctx* ctx, BatchedGroup& gr, cudaStream_t s, cudaGraph
     CK(cudaMemcpyAsync((char*)p->Bin + k * bytes, ubar[gr.fields[k]], bytes, cudaMemcpyDeviceToDevice, s));
   SolveIO io{p->Bin, p->Bout, nullptr, method_base(method), false, method_spectral(method),
              method_precond(method)};
-  ad_status st = enqueue_init<T>(ctx, p, s, io, c, &gr.n_init);
+  auto scatter = [&]() {
+    cudaError_t e = cudaSuccess;
+    for (size_t k = 0; k < gr.fields.size() && e == cudaSuccess; ++k)
+      e = cudaMemcpyAsync(u_out[gr.fields[k]], (char*)p->Bout + k * bytes, bytes, cudaMemcpyDeviceToDevice, s);
+    return e;
+  };
+  ad_status st;
+  if (solves_in_cluster(p, io.spectral, io.precond)) {
+    gr.n_init = 1;
+    if ((st = enqueue_cluster_solve<T>(ctx, p, s, io, c)) != AD_OK) return st;
+    CK(scatter());
+    return AD_OK;
+  }
+  st = enqueue_init<T>(ctx, p, s, io, c, &gr.n_init);
   if (st != AD_OK) return st;
   cudaStreamCaptureStatus cs;
   cudaGraph_t cg = nullptr;
@@ -1246,8 +1351,7 @@ ad_status capture_group(ad_ctx* ctx, BatchedGroup& gr, cudaStream_t s, cudaGraph
   if (st != AD_OK) return st;
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamEndCapture(batched body)");
   if ((st = enqueue_finish<T>(ctx, p, s, io, c, &gr.n_fin)) != AD_OK) return st;
-  for (size_t k = 0; k < gr.fields.size(); ++k)
-    CK(cudaMemcpyAsync(u_out[gr.fields[k]], (char*)p->Bout + k * bytes, bytes, cudaMemcpyDeviceToDevice, s));
+  CK(scatter());
   return AD_OK;
 }
 
@@ -1353,25 +1457,32 @@ cudaError_t issue_multi(const std::vector<MultiLaunch>& ml, cudaStream_t s) {
 }
 
 // Float32 physical-space Van Cittert, SD, CG and BiCGSTAB without a
-// preconditioner (the other variants keep one graph branch per group).
+// preconditioner (the other variants keep one graph branch per group) with at
+// least two groups too large for a cluster.
 bool multi_eligible(const BatchedEntry& be, int method) {
-  if (method_spectral(method) || method_precond(method) || be.groups.size() < 2) return false;
-  for (const BatchedGroup& gr : be.groups)
+  if (method_spectral(method) || method_precond(method)) return false;
+  size_t n = 0;
+  for (const BatchedGroup& gr : be.groups) {
     if (gr.p->f64) return false;
-  return true;
+    n += gr.p->cl.csize == 0;
+  }
+  return n >= 2;
 }
 
 ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* ubar, void* const* u_out, int method,
                               double tol, int maxit) {
-  const size_t G = be.groups.size();
+  // groups solved by clusters keep their own launch; the others share launches
+  std::vector<BatchedGroup*> big, small;
+  for (BatchedGroup& gr : be.groups) (gr.p->cl.csize ? small : big).push_back(&gr);
+  const size_t G = big.size();
   // MultiState: counters, and every group's field states
   MultiState hms{};
   hms.ngroups = (int)G;
   std::vector<FieldState*> sts(G);
   std::vector<int> cnt(G);
   for (size_t j = 0; j < G; ++j) {
-    sts[j] = be.groups[j].p->st;
-    cnt[j] = (int)be.groups[j].fields.size();
+    sts[j] = big[j]->p->st;
+    cnt[j] = (int)big[j]->fields.size();
     hms.nfields += cnt[j];
   }
   void *dms = nullptr, *dst = nullptr, *dcnt = nullptr;
@@ -1401,7 +1512,7 @@ ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* 
   std::vector<std::vector<LaunchRec>> rinit(G), rbody(G);
   ad_status st = AD_OK;
   for (size_t j = 0; j < G && st == AD_OK; ++j) {
-    Plan* p = be.groups[j].p;
+    Plan* p = big[j]->p;
     Common c;
     c.st = p->st;
     c.wait_ns = ctx->wait_ns;
@@ -1428,9 +1539,11 @@ ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* 
   if (st != AD_OK) { cudaGraphDestroy(g); return st; }
   e = cudaStreamBeginCaptureToGraph(ctx->cap, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) { cudaGraphDestroy(g); return cuda_fail(ctx, e, "cudaStreamBeginCaptureToGraph"); }
+  for (BatchedGroup* gr : small)
+    if (st == AD_OK) st = capture_group<float>(ctx, *gr, ctx->cap, 0, ubar, u_out, method, tol, maxit);
   // gather, reset the states, the initial residual of every field
   for (size_t j = 0; j < G && st == AD_OK; ++j) {
-    const BatchedGroup& gr = be.groups[j];
+    const BatchedGroup& gr = *big[j];
     const size_t bytes = (size_t)gr.p->P * sizeof(float);
     for (size_t k = 0; k < gr.fields.size() && e == cudaSuccess; ++k)
       e = cudaMemcpyAsync((char*)gr.p->Bin + k * bytes, ubar[gr.fields[k]], bytes, cudaMemcpyDeviceToDevice, ctx->cap);
@@ -1468,7 +1581,7 @@ ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* 
   // finish (CG's deferred update) and scatter, per group
   int nfin = 0;
   for (size_t j = 0; j < G && st == AD_OK; ++j) {
-    const BatchedGroup& gr = be.groups[j];
+    const BatchedGroup& gr = *big[j];
     Common c;
     c.st = gr.p->st;
     c.wait_ns = ctx->wait_ns;
@@ -1490,7 +1603,7 @@ ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* 
   be.g = g;
   be.exec = exec;
   be.multi = true;
-  be.m_init = (int)minit.size() + (int)G;
+  be.m_init = (int)minit.size() + (int)G + (int)small.size();
   be.m_body = (int)mbody.size();
   be.m_fin = nfin;
   return AD_OK;
@@ -1506,6 +1619,7 @@ ad_status build_batched(ad_ctx* ctx, BatchedEntry& be, const void* const* ubar, 
   CK(cudaGraphCreate(&g, 0));
   std::vector<cudaGraphConditionalHandle> hs(G);
   for (size_t i = 0; i < G; ++i) {
+    if (solves_in_cluster(be.groups[i].p, method_spectral(method), method_precond(method))) continue;   // no loop node
     cudaError_t e = cudaGraphConditionalHandleCreate(&hs[i], g, 1, cudaGraphCondAssignDefault);
     if (e != cudaSuccess) { cudaGraphDestroy(g); return cuda_fail(ctx, e, "cudaGraphConditionalHandleCreate"); }
   }

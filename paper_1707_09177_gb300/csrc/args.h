@@ -139,4 +139,32 @@ struct PassArgs {
                              // so the loop ends unless the last pass re-arms it
 };
 
+// One application of G inside a cluster solve: the opcodes, vectors and scalar
+// stages that the pass launches of the same application carry.
+struct ClusterStep {
+  int xf, fi, fstage, xi, ndots, istage;
+  const void *fA, *fB;
+  void *fO1, *fO2, *fO3;
+  const void *iA, *iB, *iC;
+  void *iO1, *iO2;
+};
+
+constexpr int kClusterThreads = 512;   // most threads of a CTA of k_cluster
+
+// A 2D field solved (or filtered) by one thread-block cluster (cluster.cuh).
+template <typename T>
+struct ClusterArgs {
+  PassArgs<T> a;             // geometry, filter constants, state, closure pairs (no tiles, plans or vectors)
+  FftPlan fx, fl;            // plans of the x (packed) and y axes
+  int csize;                 // CTAs per field
+  int buf;                   // complex elements of one of the three shared-memory buffers
+  int ldx, ldl;              // row strides of the x and y tiles
+  int kc;                    // sequences along y per CTA
+  float rcp_kc, rcp_own, rcp_l;
+  int n_init, n_body, n_true;
+  void* cg_u;                // CG: u and p of the deferred last update
+  const void* cg_p;
+  ClusterStep step[5];
+};
+
 }  // namespace gad

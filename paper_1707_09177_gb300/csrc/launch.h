@@ -37,6 +37,13 @@ PassKernelF fused_kernel_long(int kind, const PassArgs<float>& a);
 // against the same limit, so the opt-in is made with this margin.
 constexpr size_t kStaticSmemMargin = 4096;
 
+// A batch of small fields, one cluster of a.csize CTAs each (kernels_cluster.cu).
+template <typename T>
+cudaError_t launch_cluster(const ClusterArgs<T>& a, int batch, int threads, size_t smem, cudaStream_t s);
+// Whether the GPU can hold such a cluster.
+template <typename T>
+bool cluster_fits(int csize, int threads, size_t smem);
+
 // One pass kind over several shape groups (k_multi): `args` (device) holds
 // each group's PassArgs (vgx, vgy its own launch shape), `start` (device,
 // ngroups + 1 entries) the first block of each group; blocks = start[ngroups].

@@ -298,4 +298,49 @@ inline bool choose_pass(int L, int slots, int div, long long nseq, bool transpos
   return done();
 }
 
+// Shared-memory layout of a cluster solve (cluster.cuh): the rows of a 2D field
+// and its sequences along y spread over `csize` CTAs.
+struct ClusterShape {
+  int csize = 0, threads = 0, buf = 0, ldx = 0, ldl = 0, kc = 0;
+  size_t smem = 0;
+};
+
+constexpr size_t kClusterSmem = 224 * 1024;   // dynamic shared memory a CTA may take
+constexpr int kClusterE = 24;                 // element count whose plans have radices of at most 8
+
+// False when the grid is not one for a cluster: it takes the pass kernels.
+// Measured per pass of a single field, cluster against pass kernels: CG float32
+// 256^2 18 against 40 us; Van Cittert float64 128^2 36 against 53 us (the
+// float64 rate of 16 SMs, two lanes per clock each, is the larger part of it and
+// grows with the points). 3D fields have four more transposing steps through
+// shared memory and gain nothing (64^3 float32 CG: 53 against 50 us).
+constexpr long long kClusterPoints32 = 256 * 256, kClusterPoints64 = 128 * 128;
+
+inline bool cluster_shape(int nx, int ny, int nz, size_t csize, ClusterShape& cs) {
+  const int M = nx / 2, kxn = M + 1;
+  const long long P = (long long)nx * ny;
+  if (nz > 1 || P > (csize == 16 ? kClusterPoints64 : kClusterPoints32)) return false;
+  int rad[kMaxStages];
+  if (radices_for(M, kClusterE, rad) == 0 || radices_for(ny, kClusterE, rad) == 0) return false;
+  // as many CTAs as divide the rows, at most 16, each with at least 1024 bytes of them
+  int C = 1;
+  while (C < 16 && ny % (2 * C) == 0 && P * (long long)csize / (4 * C) >= 1024) C *= 2;
+  const int own = ny / C;
+  cs.csize = C;
+  cs.kc = (kxn + C - 1) / C;
+  cs.ldx = tile_ld(M);
+  cs.ldl = tile_ld(ny);
+  long long buf = (long long)own * cs.ldx;
+  const long long bl = (long long)cs.kc * cs.ldl, by = (long long)kxn * own;
+  if (bl > buf) buf = bl;
+  if (by > buf) buf = by;
+  const long long tabs = M / 2 + 1 + M - 1 + ny - 1;
+  const long long bytes = (3 * buf + tabs) * (long long)csize + (csize == 16 ? (long long)cs.kc * ny * 8 : 0);
+  if (bytes > (long long)kClusterSmem) return false;
+  cs.buf = (int)buf;
+  cs.smem = (size_t)bytes;
+  cs.threads = own * M > 2048 ? 512 : 256;
+  return true;
+}
+
 }  // namespace gad
