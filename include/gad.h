@@ -159,8 +159,8 @@ ad_status ad_deconvolve_host(ad_ctx* ctx, const ad_grid* grid, const void* ubar,
 /* Solves G u = u_bar for `nfields` fields of possibly different grids (2D and
  * 3D, any supported sizes, dtypes and gammas) in one call: one CUDA graph
  * whose concurrent branches each solve the fields of one grid shape (gathered
- * into a contiguous workspace, solved with their own device-side while loop,
- * scattered back). Same algorithms, stopping rules and precision as
+ * into a contiguous workspace, solved with their own device-side while loop or,
+ * small 2D grids, by one kernel, scattered back). Same algorithms, stopping rules and precision as
  * ad_deconvolve, u0 = u_bar for every field.
  *   grids      host ad_grid[nfields]
  *   ubar       host array of nfields device pointers (inputs)
@@ -246,7 +246,9 @@ ad_status ad_autotune(ad_ctx* ctx, const ad_grid* grid, int batch, ad_method met
  * back on `stream` between two CUDA events, in exactly the launch shape and
  * fused prologue/epilogue a solve uses, but on the context's internal
  * buffers (caller memory is never touched) and with every field forced
- * active and no scalar update. `index` selects the launch within the
+ * active and no scalar update. A dot pass of many blocks is timed with the
+ * small kernel that finishes its sums. Grids that a solve runs in one kernel
+ * are timed on the pass kernels all the same. `index` selects the launch within the
  * iteration body (0 .. count-1, in launch order); index = -1 only reports
  * the count; index = -2 times the whole body (all its launches in order,
  * ms_per_launch is then per body, kind and op are -1). Outputs (host, may
@@ -368,8 +370,9 @@ ad_status ad_set_wait_limit(ad_ctx* ctx, uint64_t ns);
 /* Enables (1, default) or disables (0) capture of each solve into one CUDA
  * graph whose iteration loop is a device-side conditional while node. With 0
  * the host launches the iteration body in chunks and polls the device
- * between chunks (the same iterations of Algorithms 1-4 either way). Returns
- * AD_ERR_ARG for a NULL context. */
+ * between chunks (the same iterations of Algorithms 1-4 either way). Small 2D
+ * grids (up to 256^2 points in float32, 128^2 in float64) solve in one kernel
+ * in either mode. Returns AD_ERR_ARG for a NULL context. */
 ad_status ad_set_graph_mode(ad_ctx* ctx, int enable);
 
 /* How ad_deconvolve_batched runs a batch of several shapes. 0 (default): one
@@ -379,8 +382,9 @@ ad_status ad_set_graph_mode(ad_ctx* ctx, int enable);
  * device work list of (group, field, tile) blocks; groups whose pass has
  * another per-thread element count or block size get a launch of their
  * own), one loop for the whole batch; used for float32 Van Cittert, SD, CG
- * and BiCGSTAB in physical space, every other method or precision keeps the
- * branches. The results are bitwise the same either way (each group's passes
+ * and BiCGSTAB in physical space on two or more groups too large for a
+ * one-kernel solve; every other method, precision or group keeps its
+ * branch. The results are bitwise the same either way (each group's passes
  * run in their own launch shape). Measured on the 48-field uneven batch the
  * branches are faster (the work list runs every stage until the slowest
  * field converges). Cached batched graphs are dropped. Returns AD_ERR_ARG for

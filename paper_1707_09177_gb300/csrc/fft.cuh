@@ -7,10 +7,11 @@
 // sequences held in shared memory.
 //
 // Shared-memory layout of a tile: sequence w occupies a row that starts at
-// w*ld (ld odd, in complex units); element i of the row lives at
+// w*ld (ld odd, or 16/W mod 16 for transposed float32 tiles of W < 16 rows, in
+// complex units); element i of the row lives at
 // phys(i) = i + i/16 (one pad slot every 16 elements). The pad makes the
 // power-of-two strides of the Stockham write pattern bank-conflict free, the
-// odd row stride makes column-wise (transposed) access conflict free.
+// row stride makes column-wise (transposed) access conflict free.
 #pragma once
 
 #include <cuda_runtime.h>
