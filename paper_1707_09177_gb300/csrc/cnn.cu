@@ -394,31 +394,22 @@ __global__ void k_pack_frag4t(const float* __restrict__ W4, uint2* __restrict__ 
   Wf[i] = make_uint2(pack_bf16(Bv(2 * t), Bv(2 * t + 1)), pack_bf16(Bv(2 * t + 8), Bv(2 * t + 9)));
 }
 
-// Sum of squares of each sample in float64. Bound by the float64 pipe (two
-// lanes per clock and SM), so a thread keeps four independent chains.
+// sum of squares of each sample (float64 partials per block, then per sample)
 __global__ void k_sumsq(const float* __restrict__ u, long long P, double* __restrict__ out) {
   const int b = blockIdx.y;
-  const float* ub = u + (long long)b * P;
-  double s[4] = {0.0, 0.0, 0.0, 0.0};
-  const long long st = (long long)gridDim.x * blockDim.x;
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  for (; i + 3 * st < P; i += 4 * st) {
-    float v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = ub[i + k * st];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) s[k] = fma((double)v[k], (double)v[k], s[k]);
+  double s = 0.0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
+    const double v = u[(long long)b * P + i];
+    s += v * v;
   }
-  for (; i < P; i += st) s[0] = fma((double)ub[i], (double)ub[i], s[0]);
-  double t = (s[0] + s[1]) + (s[2] + s[3]);
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   __shared__ double red[32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += red[w];
-    atomicAdd(out + b, r);
+    double t = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+    atomicAdd(out + b, t);
   }
 }
 
@@ -898,8 +889,10 @@ int cnn_tile(int X) { return X % 64 == 0 ? 64 : 32; }
 static cudaError_t launch_conv_mma(const __nv_bfloat16* in, const uint2* frag, __nv_bfloat16* out,
                                    const __nv_bfloat16* mask, int X, int Y, int Z, int B, int mode, cudaStream_t s) {
   const int TX = cnn_tile(X);
-  const size_t sm = (size_t)2 * (CONV_TY + 2) * (TX + 2) * ROWB;   // two z offsets' rows
-  const cudaError_t e = cudaFuncSetAttribute(k_conv_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  auto smem = [](int tx) { return (size_t)2 * (CONV_TY + 2) * (tx + 2) * ROWB; };   // two z offsets' rows
+  const size_t sm = smem(TX);
+  // the limit of the widest tile: the attribute is shared by every thread that launches
+  const cudaError_t e = cudaFuncSetAttribute(k_conv_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(64));
   if (e != cudaSuccess) return e;
   const dim3 g((unsigned)((X / TX) * ((Y + CONV_TY - 1) / CONV_TY)) * Z, B);
   k_conv_mma<<<g, TX / 32 * 64, sm, s>>>(in, frag, out, mask, X, Y, Z, TX, mode);
@@ -932,7 +925,7 @@ cudaError_t cnn_forward(const CnnBuffers& w, const float* ubar, float* u0, const
     return X % 64 == 0 ? launch_conv_out<64>(w, ubar, u0, X, Y, Z, B, ascale, s)
                        : launch_conv_out<32>(w, ubar, u0, X, Y, Z, B, ascale, s);
   const size_t sm = (size_t)10 * (TX + 2) * ROWB;
-  e = cudaFuncSetAttribute(k_conv_out_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  e = cudaFuncSetAttribute(k_conv_out_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, 10 * (64 + 2) * ROWB);
   if (e != cudaSuccess) return e;
   const dim3 gc((unsigned)((X / TX) * ((Y + 7) / 8)) * Z, B);
   k_conv_out_mma<<<gc, 2 * TX, sm, s>>>(w.H3, w.frag4t, ubar, w.sumsq, u0, utrue, w.sumsq + B, w.g, w.sumsq + 2 * B,
@@ -993,7 +986,8 @@ cudaError_t cnn_backward(const CnnBuffers& w, const float* ubar, int X, int Y, i
   k_reduce_parts<<<TAPS * C / 32, 256, 0, s>>>(w.part, kSmallBlocks, TAPS * C, w.grad + kW4);
   // layer 3: dW3 from (H2, dZ3); dZ2 = conv^T(dZ3, W3) masked by H2
   const size_t smw = (size_t)(WG_H * 3 * (TX + 2) + WG_Z * TX) * ROWB;
-  cudaError_t e = cudaFuncSetAttribute(k_wgrad_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw);
+  cudaError_t e = cudaFuncSetAttribute(k_wgrad_mma, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (WG_H * 3 * (64 + 2) + WG_Z * 64) * ROWB);
   if (e != cudaSuccess) return e;
   k_wgrad_mma<<<kWgradBlocks, 576, smw, s>>>(w.H2, w.dA, w.part, X, Y, Z, B, TX);
   k_reduce_parts<<<TAPS * C * C / 32, 256, 0, s>>>(w.part, kWgradBlocks, TAPS * C * C, w.grad + kW3);

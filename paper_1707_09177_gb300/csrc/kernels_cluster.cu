@@ -19,16 +19,17 @@ static cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* at, int csize, int
   return c;
 }
 
+// The same limits for every launch: they are shared by all host threads.
 template <typename T>
-static cudaError_t cluster_attributes(size_t smem) {
+static cudaError_t cluster_attributes() {
   cudaError_t e = cudaFuncSetAttribute(k_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmem);
   return e;
 }
 
 template <typename T>
 cudaError_t launch_cluster(const ClusterArgs<T>& a, int batch, int threads, size_t smem, cudaStream_t s) {
-  cudaError_t e = cluster_attributes<T>(smem);
+  cudaError_t e = cluster_attributes<T>();
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute at{};
   const cudaLaunchConfig_t c = cluster_config<T>(&at, a.csize, batch, threads, smem, s);
@@ -41,7 +42,7 @@ bool cluster_fits(int csize, int threads, size_t smem) {
   int n = 0;
   cudaLaunchAttribute at{};
   const cudaLaunchConfig_t c = cluster_config<T>(&at, csize, 1, threads, smem, nullptr);
-  const bool ok = cluster_attributes<T>(smem) == cudaSuccess &&
+  const bool ok = cluster_attributes<T>() == cudaSuccess &&
                   cudaOccupancyMaxActiveClusters(&n, k_cluster<T>, &c) == cudaSuccess && n > 0;
   if (!ok) cudaGetLastError();
   return ok;
