@@ -228,121 +228,125 @@ __global__ void __launch_bounds__(128, 3) k_conv_mma(const __nv_bfloat16* __rest
 // block marches along y: per row it stages the three z planes' rows y + 1 and
 // the dZ row y (cp.async, two rows ahead) into rings of five and three slots,
 // so a row of Hin is fetched three times (once per z plane), not nine, and its
-// latency overlaps two rows of mma. One float32 partial per tap, ci, co and
-// block. Bound by the mma.sync rate and the ldmatrix reads. Nine rows fetched
-// synchronously per output row: 64^3 x 8 1310 -> 394 us.
+// latency overlaps two rows of mma. A block writes kWgradParts float32 partials
+// per tap, ci and co, each over a part of its rows, so that the tensor cores'
+// float32 sums stay short (k_reduce_parts adds the partials in float64). Bound
+// by the mma.sync rate and the ldmatrix reads. Nine rows fetched synchronously
+// per output row: 64^3 x 8 1310 -> 394 us.
 constexpr int WG_H = 5, WG_Z = 3;          // ring slots
 __global__ void __launch_bounds__(576) k_wgrad_mma(const __nv_bfloat16* __restrict__ Hin,
-                                                      const __nv_bfloat16* __restrict__ dZ, float* __restrict__ part,
-                                                      int X, int Y, int Z, int B, int TX) {
+                                                   const __nv_bfloat16* __restrict__ dZ, float* __restrict__ part,
+                                                   int X, int Y, int Z, int B, int TX) {
   extern __shared__ __align__(16) unsigned char sm[];
   const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
   const int segs = X / TX;
   const int rstride = (TX + 2) * ROWB;
   unsigned char* dzr = sm + WG_H * 3 * rstride;
   float acc[3][4][4];
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[c][n][e] = 0.f;
   const long long P = (long long)X * Y * Z;
   const int mi = lane >> 3, li = lane & 7;
   const int wt = warp % 9, wm = warp / 9, wa = wt / 3, wb = wt - 3 * wa;
   const long long nrows = (long long)B * Z * segs * Y;
-  long long r = nrows * blockIdx.x / gridDim.x;
-  const long long rend = nrows * (blockIdx.x + 1) / gridDim.x;
   auto copy16 = [](unsigned char* dst, const __nv_bfloat16* src) {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
   };
-  while (r < rend) {
-    // a run of consecutive y of one (b, z, segment)
-    const int y0 = (int)(r % Y), n = (int)min(rend - r, (long long)(Y - y0));
-    long long col = r / Y;
-    const int x0 = (int)(col % segs) * TX;
-    col /= segs;
-    const int z = (int)(col % Z);
-    const long long base = (col / Z) * P;
-    // Hin rows y0 + i (i = -1 .. n) of the three planes, slot (i + 1) % WG_H
-    auto stage_h = [&](int i) {
-      const int y = (y0 + i + Y) % Y;
-      unsigned char* slot = sm + ((i + 1) % WG_H) * 3 * rstride;
-      for (int q = tid; q < 3 * (TX + 2) * 4; q += nthr) {
-        const int a = q / ((TX + 2) * 4), k = q - a * ((TX + 2) * 4), pt = k >> 2, ch = k & 3;
-        copy16(slot + a * rstride + pt * ROWB + ch * 16,
-               Hin + (base + ((long long)wrap(z + a - 1, Z) * Y + y) * X + wrap(x0 - 1 + pt, X)) * C + ch * 8);
-      }
-    };
-    auto stage_z = [&](int i) {
-      unsigned char* slot = dzr + (i % WG_Z) * TX * ROWB;
-      for (int q = tid; q < TX * 4; q += nthr)
-        copy16(slot + (q >> 2) * ROWB + (q & 3) * 16,
-               dZ + (base + ((long long)z * Y + y0 + i) * X + x0 + (q >> 2)) * C + (q & 3) * 8);
-    };
-    __syncthreads();                         // the previous run's rows are no longer read
-    stage_h(-1);
-    stage_h(0);
-    for (int i = 0; i < 2; ++i) {            // groups 0, 1: rows i + 1 and dZ row i
-      if (i < n) {
-        stage_h(i + 1);
-        stage_z(i);
-      }
-      asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-#pragma unroll 1
-    for (int i = 0; i < n; ++i) {
-      cp_async_wait<1>();
-      __syncthreads();                       // row i is staged; row i - 1 is no longer read
-      if (i + 2 < n) {
-        stage_h(i + 3);
-        stage_z(i + 2);
-      }
-      asm volatile("cp.async.commit_group;\n" ::: "memory");
-      const unsigned char* rowt = sm + ((i + wb) % WG_H) * 3 * rstride + wa * rstride;   // row i + wb - 1
-      const unsigned char* dzt = dzr + (i % WG_Z) * TX * ROWB;
-#pragma unroll 1
-      for (int k0 = 0; k0 < TX; k0 += 16) {
-        // B fragments (k = points, n = co) from dZ: transposed 8x8 loads.
-        // matrices: mi&1 selects k half (points k0..7 / 8..15), mi>>1 selects n tile pair
-        uint32_t bfr[4][2];
+  for (int part_i = blockIdx.x * kWgradParts; part_i < (int)(blockIdx.x + 1) * kWgradParts; ++part_i) {
+    long long r = nrows * part_i / (gridDim.x * kWgradParts);
+    const long long rend = nrows * (part_i + 1) / (gridDim.x * kWgradParts);
 #pragma unroll
-        for (int np = 0; np < 2; ++np) {
-          uint32_t rgs[4];
-          // lane address: rows = points k0 + li + 8*(mi & 1), channels 16*np + 8*(mi >> 1)
-          ldsm_x4_t(rgs, dzt + (k0 + li + 8 * (mi & 1)) * ROWB + (16 * np + 8 * (mi >> 1)) * 2);
-          bfr[2 * np + 0][0] = rgs[0];
-          bfr[2 * np + 0][1] = rgs[1];
-          bfr[2 * np + 1][0] = rgs[2];
-          bfr[2 * np + 1][1] = rgs[3];
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[c][n][e] = 0.f;
+    while (r < rend) {
+      // a run of consecutive y of one (b, z, segment)
+      const int y0 = (int)(r % Y), n = (int)min(rend - r, (long long)(Y - y0));
+      long long col = r / Y;
+      const int x0 = (int)(col % segs) * TX;
+      col /= segs;
+      const int z = (int)(col % Z);
+      const long long base = (col / Z) * P;
+      // Hin rows y0 + i (i = -1 .. n) of the three planes, slot (i + 1) % WG_H
+      auto stage_h = [&](int i) {
+        const int y = (y0 + i + Y) % Y;
+        unsigned char* slot = sm + ((i + 1) % WG_H) * 3 * rstride;
+        for (int q = tid; q < 3 * (TX + 2) * 4; q += nthr) {
+          const int a = q / ((TX + 2) * 4), k = q - a * ((TX + 2) * 4), pt = k >> 2, ch = k & 3;
+          copy16(slot + a * rstride + pt * ROWB + ch * 16,
+                 Hin + (base + ((long long)wrap(z + a - 1, Z) * Y + y) * X + wrap(x0 - 1 + pt, X)) * C + ch * 8);
         }
+      };
+      auto stage_z = [&](int i) {
+        unsigned char* slot = dzr + (i % WG_Z) * TX * ROWB;
+        for (int q = tid; q < TX * 4; q += nthr)
+          copy16(slot + (q >> 2) * ROWB + (q & 3) * 16,
+                 dZ + (base + ((long long)z * Y + y0 + i) * X + x0 + (q >> 2)) * C + (q & 3) * 8);
+      };
+      __syncthreads();                         // the previous run's rows are no longer read
+      stage_h(-1);
+      stage_h(0);
+      for (int i = 0; i < 2; ++i) {            // groups 0, 1: rows i + 1 and dZ row i
+        if (i < n) {
+          stage_h(i + 1);
+          stage_z(i);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+      }
+#pragma unroll 1
+      for (int i = 0; i < n; ++i) {
+        cp_async_wait<1>();
+        __syncthreads();                       // row i is staged; row i - 1 is no longer read
+        if (i + 2 < n) {
+          stage_h(i + 3);
+          stage_z(i + 2);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        const unsigned char* rowt = sm + ((i + wb) % WG_H) * 3 * rstride + wa * rstride;   // row i + wb - 1
+        const unsigned char* dzt = dzr + (i % WG_Z) * TX * ROWB;
+#pragma unroll 1
+        for (int k0 = 0; k0 < TX; k0 += 16) {
+          // B fragments (k = points, n = co) from dZ: transposed 8x8 loads.
+          // matrices: mi&1 selects k half (points k0..7 / 8..15), mi>>1 selects n tile pair
+          uint32_t bfr[4][2];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          // A fragments (m = ci, k = points) from the shifted input row, transposed loads:
-          // matrices 0: ci 0-7, k 0-7; 1: ci 8-15, k 0-7; 2: ci 0-7, k 8-15; 3: ci 8-15, k 8-15
-          uint32_t af[4];
-          ldsm_x4_t(af, rowt + (k0 + li + 8 * (mi >> 1) + c) * ROWB + (wm * 16 + 8 * (mi & 1)) * 2);
+          for (int np = 0; np < 2; ++np) {
+            uint32_t rgs[4];
+            // lane address: rows = points k0 + li + 8*(mi & 1), channels 16*np + 8*(mi >> 1)
+            ldsm_x4_t(rgs, dzt + (k0 + li + 8 * (mi & 1)) * ROWB + (16 * np + 8 * (mi >> 1)) * 2);
+            bfr[2 * np + 0][0] = rgs[0];
+            bfr[2 * np + 0][1] = rgs[1];
+            bfr[2 * np + 1][0] = rgs[2];
+            bfr[2 * np + 1][1] = rgs[3];
+          }
 #pragma unroll
-          for (int n4 = 0; n4 < 4; ++n4) mma_bf16(acc[c][n4], af, bfr[n4]);
+          for (int c = 0; c < 3; ++c) {
+            // A fragments (m = ci, k = points) from the shifted input row, transposed loads:
+            // matrices 0: ci 0-7, k 0-7; 1: ci 8-15, k 0-7; 2: ci 0-7, k 8-15; 3: ci 8-15, k 8-15
+            uint32_t af[4];
+            ldsm_x4_t(af, rowt + (k0 + li + 8 * (mi >> 1) + c) * ROWB + (wm * 16 + 8 * (mi & 1)) * 2);
+#pragma unroll
+            for (int n4 = 0; n4 < 4; ++n4) mma_bf16(acc[c][n4], af, bfr[n4]);
+          }
         }
       }
+      cp_async_wait<0>();
+      r += n;
     }
-    cp_async_wait<0>();
-    r += n;
-  }
-  const int g = lane >> 2, t = lane & 3;
-  float* pb = part + (long long)blockIdx.x * TAPS * C * C;
+    const int g = lane >> 2, t = lane & 3;
+    float* pb = part + (long long)part_i * TAPS * C * C;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const int tap = wt * 3 + c;
+    for (int c = 0; c < 3; ++c) {
+      const int tap = wt * 3 + c;
 #pragma unroll
-    for (int n = 0; n < 4; ++n)
+      for (int n = 0; n < 4; ++n)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int ci = wm * 16 + g + 8 * (e >> 1), co = n * 8 + 2 * t + (e & 1);
-        pb[(tap * C + ci) * C + co] = acc[c][n][e];
-      }
+        for (int e = 0; e < 4; ++e) {
+          const int ci = wm * 16 + g + 8 * (e >> 1), co = n * 8 + 2 * t + (e & 1);
+          pb[(tap * C + ci) * C + co] = acc[c][n][e];
+        }
+    }
   }
 }
 
@@ -990,7 +994,7 @@ cudaError_t cnn_backward(const CnnBuffers& w, const float* ubar, int X, int Y, i
                                        (WG_H * 3 * (64 + 2) + WG_Z * 64) * ROWB);
   if (e != cudaSuccess) return e;
   k_wgrad_mma<<<kWgradBlocks, 576, smw, s>>>(w.H2, w.dA, w.part, X, Y, Z, B, TX);
-  k_reduce_parts<<<TAPS * C * C / 32, 256, 0, s>>>(w.part, kWgradBlocks, TAPS * C * C, w.grad + kW3);
+  k_reduce_parts<<<TAPS * C * C / 32, 256, 0, s>>>(w.part, kWgradBlocks * kWgradParts, TAPS * C * C, w.grad + kW3);
   const bool tc = w.umma2 && conv_tc_shape_ok(X, Y, Z);
   if (tc) {
     if ((e = conv_tc_forward(w.dA, w.umma3t, w.dB, w.H2, X, Y, Z, B, 1, w.flag, w.wait_ns, s)) != cudaSuccess) return e;
@@ -999,7 +1003,7 @@ cudaError_t cnn_backward(const CnnBuffers& w, const float* ubar, int X, int Y, i
   }
   // layer 2: dW2 from (H1, dZ2); dZ1 = conv^T(dZ2, W2) masked by H1
   k_wgrad_mma<<<kWgradBlocks, 576, smw, s>>>(w.H1, w.dB, w.part, X, Y, Z, B, TX);
-  k_reduce_parts<<<TAPS * C * C / 32, 256, 0, s>>>(w.part, kWgradBlocks, TAPS * C * C, w.grad + kW2);
+  k_reduce_parts<<<TAPS * C * C / 32, 256, 0, s>>>(w.part, kWgradBlocks * kWgradParts, TAPS * C * C, w.grad + kW2);
   if (tc) {
     if ((e = conv_tc_forward(w.dB, w.umma2t, w.dA, w.H1, X, Y, Z, B, 1, w.flag, w.wait_ns, s)) != cudaSuccess) return e;
   } else {
