@@ -48,6 +48,7 @@ struct Plan {
   double gamma = 0.0;
   long long P = 0, SP = 0;
   PassCfg xf, xi, fl, yf, yi;
+  PassCfg xi_nodots, fl_nodots;      // xi, fl of launches without dots (plan.h)
   PassCfg sn;                        // preconditioner stencil pass (W rows per block)
   ClusterShape cl;                   // csize > 0: small grid, solved by one cluster per field (cluster.cuh)
   FftPlan clx{}, cll{};              // its plans
@@ -236,16 +237,18 @@ ad_status get_table(ad_ctx* ctx, long long L, bool f64, const void** out) {
   return AD_OK;
 }
 
-// The tile shape of a pass (plan.h) copied into its launch configuration.
-bool choose_pass(int L, int slots, int div, long long nseq, bool transposed, size_t csize, PassCfg& pc, int want_T) {
-  TileShape ts;
-  if (!gad::choose_pass(L, slots, div, nseq, transposed, csize, ts, want_T)) return false;
+// A tile shape (plan.h) as a launch configuration of `blocks` x `batch` blocks.
+PassCfg pass_cfg(const TileShape& ts, long long blocks, int batch, float rcp_a, float rcp_b) {
+  PassCfg pc;
   pc.E = ts.E;
   pc.W = ts.W;
   pc.T = ts.T;
   pc.ld = ts.ld;
   pc.smem = ts.smem;
-  return true;
+  pc.rcp_a = rcp_a;
+  pc.rcp_b = rcp_b;
+  pc.grid = dim3((unsigned)blocks, (unsigned)batch);
+  return pc;
 }
 
 // A method value: one of AD_VANCITTERT .. AD_SD, optionally OR-ed with AD_SPECTRAL.
@@ -325,14 +328,14 @@ ad_status get_plan(ad_ctx* ctx, const ad_grid* g, int batch, Plan** out) {
   // 12 elements per thread 288^3 x 3: 287 at 64, 266 at 128), filter pass at 128
   // threads (2048^2 x 16: 155 -> 139, 512^3: 284 -> 267), inverse x and y passes
   // at 256 (512^3: inverse x 337 against 344 at 128, y 211 against 225).
-  bool ok = choose_pass(M, M + 1, pow2_part(p->ny), nrow, true, cs, p->xf, M % 3 == 0 ? 128 : 64);
-  ok = ok && choose_pass(M, M + 1, pow2_part(p->ny), nrow, true, cs, p->xi, 256);
-  ok = ok && choose_pass(Lf, Lf, 0, nseq, false, cs, p->fl, 128);
-  ok = ok && (p->ndim != 3 ||
-              choose_pass(p->ny, p->ny, pow2_part(p->nz), (long long)p->kxn * p->nz, true, cs, p->yf, 256));
-  if (!ok) { delete p; return fail(ctx, AD_ERR_ARG, "no tiling for this grid"); }
+  GridTiles gt;
+  if (!grid_tiles(p->nx, p->ny, p->nz, batch, cs, gt)) {
+    delete p;
+    return fail(ctx, AD_ERR_ARG, "no tiling for this grid");
+  }
+  const int ex = plan_E(M, gt.xf.E, cs), exi = plan_E(M, gt.xi.E, cs), ef = plan_E(Lf, gt.fl.E, cs);
+  const int ey = p->ndim == 3 ? plan_E(p->ny, gt.y.E, cs) : 0;
   const void *px = nullptr, *pxi = nullptr, *pf = nullptr, *pfi = nullptr, *py = nullptr;
-  const int ex = plan_E(M, p->xf.E, cs), exi = plan_E(M, p->xi.E, cs), ef = plan_E(Lf, p->fl.E, cs), ey = plan_E(p->ny, p->yf.E, cs);
   if ((s = get_plan_table(ctx, M, ex, false, p->f64, &px)) != AD_OK ||
       (s = get_plan_table(ctx, M, exi, false, p->f64, &pxi)) != AD_OK ||
       (s = get_plan_table(ctx, Lf, ef, false, p->f64, &pf)) != AD_OK ||
@@ -341,22 +344,21 @@ ad_status get_plan(ad_ctx* ctx, const ad_grid* g, int batch, Plan** out) {
     delete p;
     return s;
   }
-  ok = make_fft(M, ex, px, p->xf.fft) && make_fft(M, exi, pxi, p->xi.fft);
-  for (PassCfg* x : {&p->xf, &p->xi}) {
-    x->rcp_a = 1.0f / (float)(p->nx / 4);
-    x->rcp_b = 1.0f / (float)(M / 2 + 1);
-    x->grid = dim3(p->ny * p->nz / x->W, batch);
-  }
-  ok = ok && make_fft(Lf, ef, pf, p->fl.fft);
-  ok = ok && make_fft(Lf, ef, pfi, p->fl.fft_inv, true);
-  p->fl.rcp_a = 1.0f / (float)(Lf / 2);
-  p->fl.rcp_b = 1.0f / (float)Lf;
-  p->fl.grid = dim3((nseq + std::max(p->fl.W, 1) - 1) / std::max(p->fl.W, 1), batch);
+  const float ra = 1.0f / (float)(p->nx / 4), rb = 1.0f / (float)(M / 2 + 1);
+  p->xf = pass_cfg(gt.xf, nrow / gt.xf.W, batch, ra, rb);
+  p->xi = pass_cfg(gt.xi, nrow / gt.xi.W, batch, ra, rb);
+  p->xi_nodots = pass_cfg(gt.xi_nodots, nrow / gt.xi_nodots.W, batch, ra, rb);
+  const float rf = 1.0f / (float)(Lf / 2), rl = 1.0f / (float)Lf;
+  p->fl = pass_cfg(gt.fl, (nseq + gt.fl.W - 1) / gt.fl.W, batch, rf, rl);
+  p->fl_nodots = pass_cfg(gt.fl_nodots, (nseq + gt.fl_nodots.W - 1) / gt.fl_nodots.W, batch, rf, rl);
+  bool ok = make_fft(M, ex, px, p->xf.fft) && make_fft(M, exi, pxi, p->xi.fft) && make_fft(Lf, ef, pf, p->fl.fft) &&
+            make_fft(Lf, ef, pfi, p->fl.fft_inv, true);
+  p->xi_nodots.fft = p->xi.fft;
+  p->fl_nodots.fft = p->fl.fft;
+  p->fl_nodots.fft_inv = p->fl.fft_inv;
   if (p->ndim == 3) {
+    p->yf = pass_cfg(gt.y, (long long)p->kxn * (p->nz / gt.y.W), batch, 1.0f / (float)(p->ny / 2), 1.0f / (float)p->ny);
     ok = ok && make_fft(p->ny, ey, py, p->yf.fft);
-    p->yf.rcp_a = 1.0f / (float)(p->ny / 2);
-    p->yf.rcp_b = 1.0f / (float)p->ny;
-    p->yf.grid = dim3(p->kxn * (p->nz / std::max(p->yf.W, 1)), batch);
     p->yi = p->yf;
   }
   if (!ok) { delete p; return fail(ctx, AD_ERR_ARG, "no tiling for this grid"); }
@@ -614,22 +616,24 @@ ad_status enqueue_G(ad_ctx* ctx, Plan* p, cudaStream_t s, const Fwd& fw, const F
     CK(issue<T>(ctx, PK_YFWD, p->yf, s, a, nl));
   }
   a.clear_cond = 0;
-  set_pass(a, p->fl);
+  const PassCfg& pf = fl.op == FI_NONE ? p->fl_nodots : p->fl;
+  set_pass(a, pf);
   a.op = fl.op;
   a.ndots = fl.op == FI_NONE ? 0 : (fl.op == FI_XGX ? 1 : 3);
   a.stage = fl.stage;
   a.inv_p = 1.0 / (double)p->P;       // Parseval: (a, b) = (1/P) sum_k a_hat conj(b_hat)
-  CK(issue<T>(ctx, PK_FILT, p->fl, s, a, nl));
+  CK(issue<T>(ctx, PK_FILT, pf, s, a, nl));
   a.ndots = 0; a.stage = SS_NONE; a.inv_p = 1.0;
   if (p->ndim == 3) {
     set_pass(a, p->yi);
     CK(issue<T>(ctx, PK_YINV, p->yi, s, a, nl));
   }
-  set_pass(a, p->xi);
+  const PassCfg& pi = iv.ndots ? p->xi : p->xi_nodots;
+  set_pass(a, pi);
   a.op = iv.op; a.A = (const T*)iv.A; a.B = (const T*)iv.B; a.C = (const T*)iv.C;
   a.O1 = (T*)iv.O1; a.O2 = (T*)iv.O2; a.O3 = nullptr;
   a.ndots = iv.ndots; a.stage = iv.stage; a.set_cond = (iv.set_cond && c.in_graph) ? 1 : 0;
-  CK(issue<T>(ctx, PK_XINV, p->xi, s, a, nl));
+  CK(issue<T>(ctx, PK_XINV, pi, s, a, nl));
   return AD_OK;
 }
 
@@ -658,9 +662,9 @@ ad_status enqueue_fwd_transform(ad_ctx* ctx, Plan* p, cudaStream_t s, const void
     set_pass(a, p->yf);
     CK(issue<T>(ctx, PK_YFWD, p->yf, s, a, nl));
   }
-  set_pass(a, p->fl);
+  set_pass(a, p->fl_nodots);
   a.O1 = (T*)out;
-  CK(issue<T>(ctx, PK_LFWD, p->fl, s, a, nl));
+  CK(issue<T>(ctx, PK_LFWD, p->fl_nodots, s, a, nl));
   return AD_OK;
 }
 
@@ -669,17 +673,17 @@ template <typename T>
 ad_status enqueue_inv_transform(ad_ctx* ctx, Plan* p, cudaStream_t s, const void* hat, void* x, int* nl) {
   Common c0;
   PassArgs<T> a = base_args<T>(p, c0);
-  set_pass(a, p->fl);
+  set_pass(a, p->fl_nodots);
   a.A = (const T*)hat;
-  CK(issue<T>(ctx, PK_LINV, p->fl, s, a, nl));
+  CK(issue<T>(ctx, PK_LINV, p->fl_nodots, s, a, nl));
   a.A = nullptr;
   if (p->ndim == 3) {
     set_pass(a, p->yi);
     CK(issue<T>(ctx, PK_YINV, p->yi, s, a, nl));
   }
-  set_pass(a, p->xi);
+  set_pass(a, p->xi_nodots);
   a.op = XI_STORE; a.O1 = (T*)x;
-  CK(issue<T>(ctx, PK_XINV, p->xi, s, a, nl));
+  CK(issue<T>(ctx, PK_XINV, p->xi_nodots, s, a, nl));
   return AD_OK;
 }
 
@@ -1034,6 +1038,7 @@ struct TileSlot {
   int L;
   int slots;
   int div;      // W must divide this (0: ragged tiles allowed)
+  int dots;     // the launches that use pc: with dots (1), without (0), all (-1)
 };
 
 void set_tile(const Plan* p, PassCfg& pc, int kind, int L, int slots, int W) {
@@ -1052,7 +1057,7 @@ void set_tile(const Plan* p, PassCfg& pc, int kind, int L, int slots, int W) {
 }
 
 template <typename T>
-double time_kind(ad_ctx* ctx, Plan* p, int method, int kind, int reps) {
+double time_kind(ad_ctx* ctx, Plan* p, int method, int kind, int dots, int reps) {
   std::vector<LaunchRec> rec;
   ctx->record = &rec;
   Common c;
@@ -1070,7 +1075,7 @@ double time_kind(ad_ctx* ctx, Plan* p, int method, int kind, int reps) {
   double total = 0.0;
   bool ok = true;
   for (LaunchRec r : rec) {
-    if (r.kind != kind) continue;
+    if (r.kind != kind || (dots >= 0 && ((r.f64 ? r.ad.ndots : r.af.ndots) > 0) != (dots > 0))) continue;
     r.af.force = r.ad.force = 1;
     r.af.stage = r.ad.stage = SS_NONE;
     r.af.set_cond = r.ad.set_cond = r.af.clear_cond = r.ad.clear_cond = 0;
@@ -1110,8 +1115,8 @@ ad_status autotune_plan(ad_ctx* ctx, Plan* p, int method, int reps) {
       trial.grid.x = (unsigned)nb;
       const PassCfg keep = p->sp;
       p->sp = trial;
-      const double ms = p->f64 ? time_kind<double>(ctx, p, method, PK_SPEC, reps)
-                               : time_kind<float>(ctx, p, method, PK_SPEC, reps);
+      const double ms = p->f64 ? time_kind<double>(ctx, p, method, PK_SPEC, -1, reps)
+                               : time_kind<float>(ctx, p, method, PK_SPEC, -1, reps);
       p->sp = keep;
       if (ms > 0.0 && (best_ms < 0.0 || ms < best_ms)) { best_ms = ms; best = trial; }
     }
@@ -1123,12 +1128,13 @@ ad_status autotune_plan(ad_ctx* ctx, Plan* p, int method, int reps) {
   }
   const int M = p->nx / 2;
   const int Lf = p->ndim == 3 ? p->nz : p->ny;
-  std::vector<TileSlot> slots = {{&p->xf, PK_XFWD, M, M + 1, pow2_part(p->ny)},
-                                 {&p->xi, PK_XINV, M, M + 1, pow2_part(p->ny)},
-                                 {&p->fl, PK_FILT, Lf, Lf, 0}};
+  std::vector<TileSlot> slots = {{&p->xf, PK_XFWD, M, M + 1, pow2_part(p->ny), -1},
+                                 {&p->xi, PK_XINV, M, M + 1, pow2_part(p->ny), 1},
+                                 {&p->fl, PK_FILT, Lf, Lf, 0, 1},
+                                 {&p->fl_nodots, PK_FILT, Lf, Lf, 0, 0}};
   if (p->ndim == 3) {
-    slots.push_back({&p->yf, PK_YFWD, p->ny, p->ny, pow2_part(p->nz)});
-    slots.push_back({&p->yi, PK_YINV, p->ny, p->ny, pow2_part(p->nz)});
+    slots.push_back({&p->yf, PK_YFWD, p->ny, p->ny, pow2_part(p->nz), -1});
+    slots.push_back({&p->yi, PK_YINV, p->ny, p->ny, pow2_part(p->nz), -1});
   }
   const size_t cs = p->f64 ? 16 : 8;
   for (TileSlot& sl : slots) {
@@ -1146,8 +1152,8 @@ ad_status autotune_plan(ad_ctx* ctx, Plan* p, int method, int reps) {
       if ((sl.kind == PK_XINV || sl.kind == PK_FILT) && trial.grid.x > p->maxblk) continue;
       const PassCfg keep = *sl.pc;
       *sl.pc = trial;
-      const double ms = p->f64 ? time_kind<double>(ctx, p, method, sl.kind, reps)
-                               : time_kind<float>(ctx, p, method, sl.kind, reps);
+      const double ms = p->f64 ? time_kind<double>(ctx, p, method, sl.kind, sl.dots, reps)
+                               : time_kind<float>(ctx, p, method, sl.kind, sl.dots, reps);
       *sl.pc = keep;
       if (ms > 0.0 && (best_ms < 0.0 || ms < best_ms)) { best_ms = ms; best = trial; }
     }

@@ -230,10 +230,14 @@ inline bool choose_tile(int L, int E, int slots, int div, size_t csize, TileShap
   return true;
 }
 
-// Blocks per field below which a pass cannot fill the GPU with the default
-// tile, and complex elements per field below which even 16 elements per
-// thread leave most of the 152 SMs' warp slots empty.
+// Blocks below which a launch cannot fill the GPU with the default tile: of one
+// field where it has dots, of all its fields where it has none; and complex
+// elements per field below which even 16 elements per thread leave most of
+// the 152 SMs' warp slots empty. Two blocks per SM for the launches without
+// dots: with one, 32 fields of 192^2 float64 filter in 259 us, with two in 198,
+// with four 64^3 float32 x 4 takes 54 against 51 us.
 constexpr int kWantBlocks = 152;
+constexpr int kWantLaunch = 2 * 152;
 constexpr long long kSmallElems = 152 * 64 * 16;
 
 // Row stride of a tile of W rows that is stored or loaded transposed (the W
@@ -250,15 +254,20 @@ inline int transposed_ld(int ld, int W, size_t csize) {
 }
 
 // Elements per thread and tile of a pass over `nseq` sequences of length L
-// per field. Default: 12 (fused_length) or pick_E(L) and choose_tile's 256-thread blocks, for
-// every grid that gives kWantBlocks of them. Smaller grids get narrower
-// tiles, the widest that still gives kWantBlocks, down to rows of 32 bytes
-// (one sector) in the transposed spectra and to one warp; grids under
-// kSmallElems also get small_E(L). The rule looks at one field, never at the
-// batch: the tile fixes the order of the dot sums, and a field's result must
-// not depend on the batch it is solved in.
+// per field. Default: 12 (fused_length) or pick_E(L) elements and choose_tile's
+// blocks narrowed to about `want_T` threads. Small grids get small_E(L) and
+// narrower tiles, the widest that still gives enough blocks, down to rows of 32
+// bytes (one sector) in the transposed spectra and to one warp.
+// A field's result must not depend on the batch it is solved in. The element
+// count (it sets the radices and with them the rounding) and the tile of a
+// launch with dots (it sets the order of their sums) therefore follow the
+// field alone; `batch` = 0 asks for that tile. The tile of a launch without
+// dots changes no result and follows the blocks of all its `batch` fields:
+// narrow tiles cost a launch that fills the GPU without them (float64 closure
+// of four 72 x 72 x 96 velocities 2.81 ms with the field's tiles, 2.60 with the
+// launch's, filter of 32 fields 96 x 72 x 72 3.79 and 3.54 ms).
 inline bool choose_pass(int L, int slots, int div, long long nseq, bool transposed, size_t csize, TileShape& ts,
-                        int want_T = 256) {
+                        int want_T = 256, int batch = 0) {
   const int E0 = csize == 8 && fused_length(L) && !(transposed && L > 768) ? 12 : pick_E(L);
   if (!choose_tile(L, E0, slots, div, csize, ts)) return false;
   auto done = [&]() {
@@ -274,10 +283,15 @@ inline bool choose_pass(int L, int slots, int div, long long nseq, bool transpos
     ts.T /= 2;
     ts.smem /= 2;
   }
-  if ((nseq + ts.W - 1) / ts.W >= kWantBlocks) return done();
+  auto enough = [&](int W) {
+    const long long n = (nseq + W - 1) / W;
+    return batch > 0 ? n * batch >= kWantLaunch : n >= kWantBlocks;
+  };
   int rad[kMaxStages];
   int E = E0;
-  if (nseq * L < kSmallElems && radices_for(L, small_E(L), rad) > 0) E = small_E(L);
+  if ((nseq + ts.W - 1) / ts.W < kWantBlocks && nseq * L < kSmallElems && radices_for(L, small_E(L), rad) > 0)
+    E = small_E(L);
+  if (E == E0 && enough(ts.W)) return done();
   TileShape best;
   for (int W = 4096; W >= 1; W /= 2) {
     if (div > 0 && div % W != 0) continue;
@@ -292,10 +306,27 @@ inline bool choose_pass(int L, int slots, int div, long long nseq, bool transpos
     best.T = (int)(tot / E);
     best.ld = ts.ld;
     best.smem = smem;
-    if ((nseq + W - 1) / W >= kWantBlocks) break;
+    if (enough(W) && (batch == 0 || best.T <= want_T)) break;
   }
   if (best.W) ts = best;
   return done();
+}
+
+// The tiles of every pass of a grid: forward x, inverse x and filter with and
+// without dots, both y passes (3D).
+struct GridTiles {
+  TileShape xf, xi, xi_nodots, fl, fl_nodots, y;
+};
+
+inline bool grid_tiles(int nx, int ny, int nz, int batch, size_t csize, GridTiles& t) {
+  const int M = nx / 2, kxn = M + 1, L = nz > 1 ? nz : ny, dx = pow2_part(ny);
+  const long long rows = (long long)ny * nz, seqs = nz > 1 ? (long long)kxn * ny : kxn;
+  return choose_pass(M, M + 1, dx, rows, true, csize, t.xf, M % 3 == 0 ? 128 : 64, batch) &&
+         choose_pass(M, M + 1, dx, rows, true, csize, t.xi, 256) &&
+         choose_pass(M, M + 1, dx, rows, true, csize, t.xi_nodots, 256, batch) &&
+         choose_pass(L, L, 0, seqs, false, csize, t.fl, 128) &&
+         choose_pass(L, L, 0, seqs, false, csize, t.fl_nodots, 128, batch) &&
+         (nz == 1 || choose_pass(ny, ny, pow2_part(nz), (long long)kxn * nz, true, csize, t.y, 256, batch));
 }
 
 // Shared-memory layout of a cluster solve (cluster.cuh): the rows of a 2D field
