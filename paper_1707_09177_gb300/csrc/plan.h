@@ -37,8 +37,14 @@ inline int pick_E(int L) { return (L % 3 == 0) ? 24 : 16; }
 constexpr int kMaxStages = 5;       // the kernels unroll at most 5 stages
 
 // Elements per FFT thread on a grid too small to fill the GPU (choose_pass):
-// four to six times as many threads, each with a shorter chain.
-inline int small_E(int L) { return (L % 3 == 0) ? 12 : 4; }
+// two or four times as many threads, each with a shorter chain; 0: the default.
+// A batch of the same grid takes the same count (see choose_pass), so it must
+// not be the slower one there. 12 elements, and 4 in float64, whose passes are
+// bound by arithmetic, are not; float32 passes of powers of two are bound by
+// shared memory, which the radices of 4 elements (4 and 2) pass through up to
+// twice as often: one 64^3 field filters in 39 us with 4 elements and in 51 with
+// 16, but 64 of them in 279 and 237, 32 fields of 512^2 in 136 and 72.
+inline int small_E(int L, size_t csize) { return (L % 3 == 0) ? 12 : csize == 16 ? 4 : 0; }
 
 // Balanced radix list for a length L and E elements per thread: the factors 3
 // first, then the power of two split into as few stages of at most 2^4 (E =
@@ -231,14 +237,18 @@ inline bool choose_tile(int L, int E, int slots, int div, size_t csize, TileShap
 }
 
 // Blocks below which a launch cannot fill the GPU with the default tile: of one
-// field where it has dots, of all its fields where it has none; and complex
-// elements per field below which even 16 elements per thread leave most of
-// the 152 SMs' warp slots empty. Two blocks per SM for the launches without
-// dots: with one, 32 fields of 192^2 float64 filter in 259 us, with two in 198,
-// with four 64^3 float32 x 4 takes 54 against 51 us.
+// field where it has dots, of all its fields where it has none. Two blocks per
+// SM for the launches without dots: with one, 32 fields of 192^2 float64 filter
+// in 259 us, with two in 198, with four 64^3 float32 x 4 takes 54 against 51 us.
 constexpr int kWantBlocks = 152;
 constexpr int kWantLaunch = 2 * 152;
-constexpr long long kSmallElems = 152 * 64 * 16;
+// Complex elements per field below which a pass takes small_E: with the default
+// count less than a third of the GPU's threads would have work. For powers of
+// two (float64) a quarter of that: one 64^3 field (135,168 elements) filters in
+// 68 us with 4 elements and 111 with 16, but the closure of 32 such velocities
+// takes 6.6 against 6.1 ms; 256^2 (33,024): 39 against 88 us for one, 2.10
+// against 1.93 ms for 256 (2.06 before narrow tiles).
+constexpr long long kSmallElems = 152 * 64 * 16, kSmallElemsPow2 = kSmallElems / 4;
 
 // Row stride of a tile of W rows that is stored or loaded transposed (the W
 // values of one wavenumber by consecutive threads): the 128 bytes that a
@@ -289,8 +299,9 @@ inline bool choose_pass(int L, int slots, int div, long long nseq, bool transpos
   };
   int rad[kMaxStages];
   int E = E0;
-  if ((nseq + ts.W - 1) / ts.W < kWantBlocks && nseq * L < kSmallElems && radices_for(L, small_E(L), rad) > 0)
-    E = small_E(L);
+  if ((nseq + ts.W - 1) / ts.W < kWantBlocks && nseq * L < (L % 3 == 0 ? kSmallElems : kSmallElemsPow2) &&
+      small_E(L, csize) > 0 && radices_for(L, small_E(L, csize), rad) > 0)
+    E = small_E(L, csize);
   if (E == E0 && enough(ts.W)) return done();
   TileShape best;
   for (int W = 4096; W >= 1; W /= 2) {

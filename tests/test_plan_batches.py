@@ -74,3 +74,16 @@ def test_a_full_launch_has_no_narrow_tiles(tiles):
     # the filter pass of a batch of 96 x 72 x 72 float64 fields
     assert tiles[(96, 72, 72), 16, 16]["fl_nodots"][2] >= 96
     assert tiles[(96, 72, 72), 16, 1]["fl"][2] < 96
+
+
+def test_few_elements_per_thread_only_where_a_batch_gains_too(tiles):
+    """4 elements per thread (radices 4 and 2) in float64 on small grids only:
+    batches of float32 fields and of larger float64 ones are slower with them."""
+    for (grid, cs, batch), r in tiles.items():
+        if not r["ok"]:
+            continue
+        for k, kx in (("xf", grid[0] // 2), ("xi", grid[0] // 2), ("fl", grid[0] // 2 + 1), ("y", grid[0] // 2 + 1)):
+            if r[k][0] == 4:
+                assert cs == 16 and kx * grid[1] * grid[2] < 152 * 16 * 16, (grid, cs, k)
+    assert tiles[(512, 512, 1), 8, 16]["fl"][0] == tiles[(64, 64, 64), 8, 1]["fl"][0] == 16
+    assert tiles[(256, 256, 1), 16, 1]["fl"][0] == 4 and tiles[(64, 64, 64), 16, 1]["fl"][0] == 16
