@@ -30,6 +30,12 @@
  *   - No entry point throws. Arguments are checked before any launch; an
  *     error returns a negative status and leaves outputs unspecified.
  *   - A context is not thread safe; use one context per host thread.
+ *   - A field's result does not depend on the other fields of its call. On 2D
+ *     grids of up to 256^2 points (float32) or 128^2 (float64) it may differ in
+ *     its last bits between calls of few and of many such fields: up to as
+ *     many as the GPU runs at once (14 of the largest) are filtered, and solved
+ *     by Algorithms 1-4 in physical space, by one kernel that adds in another
+ *     order. Elsewhere a field's result is the same bits in every batch.
  */
 #ifndef GAD_H
 #define GAD_H
@@ -160,8 +166,8 @@ ad_status ad_deconvolve_host(ad_ctx* ctx, const ad_grid* grid, const void* ubar,
  * 3D, any supported sizes, dtypes and gammas) in one call: one CUDA graph
  * whose concurrent branches each solve the fields of one grid shape (gathered
  * into a contiguous workspace, solved with their own device-side while loop or,
- * small 2D grids, by one kernel, scattered back). Same algorithms, stopping rules and precision as
- * ad_deconvolve, u0 = u_bar for every field.
+ * few small 2D fields, by one kernel, scattered back). Same algorithms, stopping
+ * rules and precision as ad_deconvolve, u0 = u_bar for every field.
  *   grids      host ad_grid[nfields]
  *   ubar       host array of nfields device pointers (inputs)
  *   u_out      host array of nfields device pointers (outputs, no aliasing)
@@ -370,9 +376,8 @@ ad_status ad_set_wait_limit(ad_ctx* ctx, uint64_t ns);
 /* Enables (1, default) or disables (0) capture of each solve into one CUDA
  * graph whose iteration loop is a device-side conditional while node. With 0
  * the host launches the iteration body in chunks and polls the device
- * between chunks (the same iterations of Algorithms 1-4 either way). Small 2D
- * grids (up to 256^2 points in float32, 128^2 in float64) solve in one kernel
- * in either mode. Returns AD_ERR_ARG for a NULL context. */
+ * between chunks (the same iterations of Algorithms 1-4 either way). Few
+ * fields of a small 2D grid (see above) solve in one kernel in either mode. Returns AD_ERR_ARG for a NULL context. */
 ad_status ad_set_graph_mode(ad_ctx* ctx, int enable);
 
 /* How ad_deconvolve_batched runs a batch of several shapes. 0 (default): one

@@ -38,17 +38,17 @@ cudaError_t launch_cluster(const ClusterArgs<T>& a, int batch, int threads, size
 }
 
 template <typename T>
-bool cluster_fits(int csize, int threads, size_t smem) {
+int cluster_room(int csize, int threads, size_t smem) {
   int n = 0;
   cudaLaunchAttribute at{};
   const cudaLaunchConfig_t c = cluster_config<T>(&at, csize, 1, threads, smem, nullptr);
   const bool ok = cluster_attributes<T>() == cudaSuccess &&
                   cudaOccupancyMaxActiveClusters(&n, k_cluster<T>, &c) == cudaSuccess && n > 0;
   if (!ok) cudaGetLastError();
-  return ok;
+  return ok ? n : 0;
 }
 
 template cudaError_t launch_cluster<GAD_REAL>(const ClusterArgs<GAD_REAL>&, int, int, size_t, cudaStream_t);
-template bool cluster_fits<GAD_REAL>(int, int, size_t);
+template int cluster_room<GAD_REAL>(int, int, size_t);
 
 }  // namespace gad

@@ -40,9 +40,9 @@ constexpr size_t kStaticSmemMargin = 4096;
 // A batch of small fields, one cluster of a.csize CTAs each (kernels_cluster.cu).
 template <typename T>
 cudaError_t launch_cluster(const ClusterArgs<T>& a, int batch, int threads, size_t smem, cudaStream_t s);
-// Whether the GPU can hold such a cluster.
+// How many such clusters the GPU holds at a time.
 template <typename T>
-bool cluster_fits(int csize, int threads, size_t smem);
+int cluster_room(int csize, int threads, size_t smem);
 
 // One pass kind over several shape groups (k_multi): `args` (device) holds
 // each group's PassArgs (vgx, vgy its own launch shape), `start` (device,
