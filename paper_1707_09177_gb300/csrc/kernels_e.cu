@@ -23,10 +23,8 @@ cudaError_t launch_pass_e(int kind, dim3 grid, int threads, size_t smem, cudaStr
   if constexpr (sizeof(T) == 4 && E == 12) {
     if (auto fk = fused_kernel(kind, a)) fn = fk;
   }
-  if (smem + kStaticSmemMargin > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(fn, smem, kPassSmem);
+  if (e != cudaSuccess) return e;
   fn<<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }

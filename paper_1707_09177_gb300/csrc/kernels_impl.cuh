@@ -18,10 +18,8 @@ cudaError_t launch_pass(int kind, int E, dim3 grid, int threads, size_t smem, cu
                         const PassArgs<T>& a) {
   if (kind == PK_SPEC) return launch_spec<T>(grid, s, a);
   if (kind == PK_STEN) {
-    if (smem + kStaticSmemMargin > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(k_sten<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(k_sten<T>, smem, kMaxSmem);
+    if (e != cudaSuccess) return e;
     k_sten<T><<<grid, threads, smem, s>>>(a);
     return cudaGetLastError();
   }
@@ -52,10 +50,8 @@ template <typename T>
 cudaError_t launch_shell(const void* X, int nx, int ny, int nz, long long SP, int batch, int ncomp, int nbins,
                          double scale, double* out, cudaStream_t s) {
   const size_t smem = (size_t)nbins * sizeof(double);
-  if (smem + kStaticSmemMargin > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_shell<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(k_shell<T>, smem, kMaxSmem);
+  if (e != cudaSuccess) return e;
   long long bx = (SP + 1023) / 1024;
   bx = std::min<long long>(bx, std::max<long long>(1, (1216 + batch - 1) / batch));
   k_shell<T><<<dim3((unsigned)std::max<long long>(bx, 1), batch), 256, smem, s>>>(
@@ -67,10 +63,8 @@ template <typename T>
 cudaError_t launch_hist(const T* x, long long n, double lo, double scale, int nbins, unsigned long long* counts,
                         cudaStream_t s) {
   const size_t smem = (size_t)(nbins + 3) * sizeof(unsigned);
-  if (smem + kStaticSmemMargin > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_hist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(k_hist<T>, smem, kMaxSmem);
+  if (e != cudaSuccess) return e;
   const long long blocks = std::max<long long>(1, std::min<long long>((n + 2047) / 2048, 1216));
   k_hist<T><<<(unsigned)blocks, 256, smem, s>>>(x, n, (T)lo, (T)scale, nbins, counts);
   return cudaGetLastError();

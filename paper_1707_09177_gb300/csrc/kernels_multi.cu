@@ -12,10 +12,8 @@ namespace gad {
 template <typename T, int E, int KIND>
 static cudaError_t launch_multi_k(int blocks, int threads, size_t smem, cudaStream_t s, const PassArgs<T>* args,
                                   const int* start, int ngroups) {
-  if (smem + kStaticSmemMargin > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_multi<T, E, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(k_multi<T, E, KIND>, smem, kPassSmem);
+  if (e != cudaSuccess) return e;
   k_multi<T, E, KIND><<<blocks, threads, smem, s>>>(args, start, ngroups);
   return cudaGetLastError();
 }

@@ -34,8 +34,19 @@ PassKernelF fused_kernel_long(int kind, const PassArgs<float>& a);
 
 // Dynamic shared memory above 48 KB per block needs an opt-in; the kernels'
 // static shared memory (reduction scratch, mbarrier: under 1 KB) counts
-// against the same limit, so the opt-in is made with this margin.
+// against the same limit, so the opt-in is made with this margin. The limit
+// belongs to the kernel and is shared by all host threads, so every launch
+// sets the same one, the most that a kernel of its kind may take: a launch that
+// set its own size could lower it between another thread's opt-in and launch.
 constexpr size_t kStaticSmemMargin = 4096;
+constexpr size_t kPassSmem = 104 * 1024;      // tiles: 100 KB and the padding of transposed_ld (plan.h)
+constexpr size_t kMaxSmem = 224 * 1024;       // what a block may take beside its static shared memory
+
+template <typename Fn>
+cudaError_t allow_smem(Fn* fn, size_t smem, size_t most) {
+  if (smem + kStaticSmemMargin <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
 
 // A batch of small fields, one cluster of a.csize CTAs each (kernels_cluster.cu).
 template <typename T>
