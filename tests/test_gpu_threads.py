@@ -30,8 +30,8 @@ def _spin(lib, gad, torch, nx, batch, dtype, calls, start, out):
     lib.ad_destroy(ctx)
 
 
-# inverse x passes of 52,352 and 49,792 bytes (float32), of 88,704 and 66,176 (float64)
-@pytest.mark.parametrize("case", [("f32", 3072, 160, 2916, 160), ("f64", 2592, 160, 3888, 80)])
+# inverse x passes of 52,352 and 52,232 bytes (float32), of 78,464 and 52,352 (float64)
+@pytest.mark.parametrize("case", [("f32", 3072, 160, 12288, 40), ("f64", 2304, 160, 3072, 80)])
 def test_two_threads_with_their_own_contexts(gad, case):
     import torch
     dtype = torch.float64 if case[0] == "f64" else torch.float32
