@@ -530,6 +530,20 @@ __global__ void __launch_bounds__(128, 3) k_conv_1ch(const float* __restrict__ S
 }
 constexpr size_t kConv1Smem = 4 * 4 * (32 * ROWB + 64);
 
+// sum_tap, ci W4[tap][ci] H3[p + off(tap)][ci] of one point, weights rounded to
+// bfloat16 as in the matrix products.
+__device__ __noinline__ float out_point(const __nv_bfloat16* H3, const float* W4, long long base, int x, int y, int z,
+                                        int X, int Y, int Z) {
+  float s = 0.f;
+  for (int tap = 0; tap < TAPS; ++tap) {
+    const long long q = base + ((long long)wrap(z + tap / 9 - 1, Z) * Y + wrap(y + tap / 3 % 3 - 1, Y)) * X +
+                        wrap(x + tap % 3 - 1, X);
+    for (int ci = 0; ci < C; ++ci)
+      s = fmaf(__bfloat162float(__float2bfloat16_rn(W4[tap * C + ci])), __bfloat162float(H3[q * C + ci]), s);
+  }
+  return s;
+}
+
 // Layer 4 of a training step, with the loss and its gradient: the implicit GEMM
 // of k_conv_mma with one n8 tile whose eight columns are eight output rows y0 ..
 // y0+7. A staged row d (relative to y0) is multiplied once by the fragment
@@ -538,12 +552,15 @@ constexpr size_t kConv1Smem = 4 * 4 * (32 * ROWB + 64);
 // column per output row took 432. Every output still adds its 27 taps x two
 // halves of 16 channels in that order (the zero columns add nothing), which
 // the loss gradient, proportional to the small difference u0 - u_true, is
-// sensitive to. A block owns a TX-point x-segment, a warp 16 of its points.
-// 64^3 x 8: 402 -> 225 us.
+// sensitive to. Where a staged activation is not finite its products with the
+// zero columns are not zero; a sum that is not finite is therefore formed again
+// from the output's own taps (out_point). A block owns a TX-point x-segment, a
+// warp 16 of its points. 64^3 x 8: 402 -> 225 us.
 // It writes u0, g = sigma * A * 2 (u0 - u_true) / ||u_true||^2 / B and
 // accumulates sum (u0 - u_true)^2 / ||u_true||^2 / B into loss.
 __global__ void __launch_bounds__(128) k_conv_out_mma(const __nv_bfloat16* __restrict__ H3,
-                                                      const uint2* __restrict__ Wf, const float* __restrict__ ubar,
+                                                      const uint2* __restrict__ Wf, const float* __restrict__ W4,
+                                                      const float* __restrict__ ubar,
                                                       const double* __restrict__ sumsq, float* __restrict__ u0,
                                                       const float* __restrict__ utrue,
                                                       const double* __restrict__ tsumsq, float* __restrict__ gout,
@@ -590,8 +607,10 @@ __global__ void __launch_bounds__(128) k_conv_out_mma(const __nv_bfloat16* __res
   for (int e = 0; e < 4; ++e) {              // point g + 8 (e / 2), row 2t + e % 2
     const int y = y0 + 2 * t + (e & 1);
     if (y < Y) {
-      const long long gi = base + ((long long)z * Y + y) * X + x0 + warp * 16 + g + 8 * (e >> 1);
-      const float uo = ubar[gi] + (float)sigma * acc[e];
+      const int x = x0 + warp * 16 + g + 8 * (e >> 1);
+      const long long gi = base + ((long long)z * Y + y) * X + x;
+      const float o = isfinite(acc[e]) ? acc[e] : out_point(H3, W4, base, x, y, z, X, Y, Z);
+      const float uo = ubar[gi] + (float)sigma * o;
       u0[gi] = uo;
       const double df = (double)uo - (double)utrue[gi];
       lsum += df * df * inv;
@@ -932,8 +951,8 @@ cudaError_t cnn_forward(const CnnBuffers& w, const float* ubar, float* u0, const
   e = cudaFuncSetAttribute(k_conv_out_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, 10 * (64 + 2) * ROWB);
   if (e != cudaSuccess) return e;
   const dim3 gc((unsigned)((X / TX) * ((Y + 7) / 8)) * Z, B);
-  k_conv_out_mma<<<gc, 2 * TX, sm, s>>>(w.H3, w.frag4t, ubar, w.sumsq, u0, utrue, w.sumsq + B, w.g, w.sumsq + 2 * B,
-                                        X, Y, Z, B, TX, ascale);
+  k_conv_out_mma<<<gc, 2 * TX, sm, s>>>(w.H3, w.frag4t, w.master + kW4, ubar, w.sumsq, u0, utrue, w.sumsq + B, w.g,
+                                        w.sumsq + 2 * B, X, Y, Z, B, TX, ascale);
   return cudaGetLastError();
 }
 
