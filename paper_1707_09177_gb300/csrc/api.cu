@@ -1950,10 +1950,10 @@ ad_status ad_guess_infer(ad_ctx* ctx, const ad_grid* grid, const float* weights,
   if ((s = get_cnn(ctx, grid, batch, false, &cw)) != AD_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
   CK(cudaMemcpyAsync(cw->w.master, weights, sizeof(float) * kCnnWeights, cudaMemcpyDeviceToDevice, st));
-  CK(cnn_pack(cw->w, st));
+  CK(cnn_pack(cw->w, false, st));
   CK(cnn_forward(cw->w, ubar, u0, nullptr, (int)grid->n[0], (int)grid->n[1], (int)grid->n[2], batch,
                  cnn_ascale(grid->gamma), st));
-  ctx->launches = 5 + 5 + 1 + (cw->w.umma2 ? 4 : 0);
+  ctx->launches = 5 + 5 + (cw->w.umma2 ? 4 : 0);     // packing, sum of squares and four layers
   // the tensor-core path reports a bounded wait that gave up
   if (cw->w.umma2) return cnn_flag_status(ctx, cw, st);
   return AD_OK;
@@ -1974,7 +1974,7 @@ ad_status ad_guess_time_conv(ad_ctx* ctx, const ad_grid* grid, int batch, int re
   // defined inputs: zero weights and activations (the timing does not depend on the values)
   CK(cudaMemsetAsync(cw->w.master, 0, sizeof(float) * kCnnWeights, st));
   CK(cudaMemsetAsync(cw->w.H1, 0, act, st));
-  CK(cnn_pack(cw->w, st));
+  CK(cnn_pack(cw->w, false, st));
   bool tc = false;
   CK(cnn_conv_layer(cw->w, X, Y, Z, batch, st, &tc));          // warm-up
   cudaEvent_t e0, e1;
@@ -2008,7 +2008,7 @@ ad_status ad_guess_grad(ad_ctx* ctx, const ad_grid* grid, const float* weights, 
   cudaStream_t st = (cudaStream_t)stream;
   const int X = (int)grid->n[0], Y = (int)grid->n[1], Z = (int)grid->n[2];
   CK(cudaMemcpyAsync(cw->w.master, weights, sizeof(float) * kCnnWeights, cudaMemcpyDeviceToDevice, st));
-  CK(cnn_pack(cw->w, st));
+  CK(cnn_pack(cw->w, true, st));
   CK(cnn_forward(cw->w, ubar, cw->u0, utrue, X, Y, Z, batch, cnn_ascale(grid->gamma), st));
   CK(cnn_backward(cw->w, ubar, X, Y, Z, batch, st));
   CK(cudaMemcpyAsync(grad, cw->w.grad, sizeof(float) * kCnnWeights, cudaMemcpyDeviceToDevice, st));
@@ -2058,7 +2058,7 @@ ad_status ad_guess_train(ad_ctx* ctx, const ad_grid* grid, int npairs, const flo
         CK(cudaMemcpyAsync(cw->ub + k * P, ubar + src, sizeof(float) * P, cudaMemcpyDeviceToDevice, st));
         CK(cudaMemcpyAsync(cw->ut + k * P, utrue + src, sizeof(float) * P, cudaMemcpyDeviceToDevice, st));
       }
-      CK(cnn_pack(cw->w, st));
+      CK(cnn_pack(cw->w, true, st));
       CK(cnn_forward(cw->w, cw->ub, cw->u0, cw->ut, X, Y, Z, batch, cnn_ascale(grid->gamma), st));
       CK(cnn_backward(cw->w, cw->ub, X, Y, Z, batch, st));
       CK(cnn_adam(cw->w, ++step, (float)lr, st));

@@ -755,8 +755,7 @@ template <int TX>
 static cudaError_t launch_conv_out(const CnnBuffers& w, const float* ubar, float* u0, int X, int Y, int Z, int B,
                                    double ascale, cudaStream_t s) {
   const long long cols = (long long)(X / TX) * ((Y + OUT_TY - 1) / OUT_TY);
-  int zc = Z;       // planes per block: at least four waves of three blocks per SM, and at least 8 planes (halo 2 of 10)
-  while (zc > 8 && cols * B * ((Z + zc - 1) / zc) < 4 * 3 * 152) zc = (zc + 1) / 2;
+  const int zc = out_planes(cols * B, Z);
   const cudaError_t e =
       cudaFuncSetAttribute(k_conv_out<TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OutTile<TX>::smem);
   if (e != cudaSuccess) return e;
@@ -965,14 +964,16 @@ cudaError_t cnn_conv_layer(const CnnBuffers& w, int X, int Y, int Z, int B, cuda
   return launch_conv_mma(w.H1, w.frag2, w.H2, nullptr, X, Y, Z, B, 0, s);
 }
 
-cudaError_t cnn_pack(const CnnBuffers& w, cudaStream_t s) {
+cudaError_t cnn_pack(const CnnBuffers& w, bool training, cudaStream_t s) {
   const int n = TAPS * 2 * 4 * 32;
   k_pack_frag<<<(n + 255) / 256, 256, 0, s>>>(w.master + kW2, w.frag2, 0);
   k_pack_frag<<<(n + 255) / 256, 256, 0, s>>>(w.master + kW3, w.frag3, 0);
   k_pack_frag<<<(n + 255) / 256, 256, 0, s>>>(w.master + kW2, w.frag2t, 1);
   k_pack_frag<<<(n + 255) / 256, 256, 0, s>>>(w.master + kW3, w.frag3t, 1);
-  k_pack_frag4<<<1, 256, 0, s>>>(w.master + kW4, w.frag4);
-  k_pack_frag4t<<<(180 * 32 + 255) / 256, 256, 0, s>>>(w.master + kW4, w.frag4t);
+  if (training)
+    k_pack_frag4t<<<(180 * 32 + 255) / 256, 256, 0, s>>>(w.master + kW4, w.frag4t);
+  else
+    k_pack_frag4<<<1, 256, 0, s>>>(w.master + kW4, w.frag4);
   if (w.umma2) {
     cudaError_t e;
     if ((e = conv_tc_pack(w.master + kW2, w.umma2, 0, s)) != cudaSuccess ||

@@ -50,8 +50,23 @@ constexpr long long kCnnPartFloats = (long long)kWgradBlocks * kWgradParts * 27 
                                          ? (long long)kWgradBlocks * kWgradParts * 27 * 32 * 32
                                          : (long long)kSmallBlocks * 27 * 32;
 
+// Output planes per block of k_conv_out, of Z planes over `columns` (x segments
+// x y tiles x fields); a block reads two planes more than it writes. At least
+// four waves of three blocks per SM where that leaves 8 planes or more; below a
+// block per SM the march of one block is all the time there is, and it gets as
+// short as one plane (inference of one 24 x 24 x 32 field: 9 blocks of 8 planes
+// 85 us, 72 of one 79; a layer-4 packing launch less is part of that).
+inline int out_planes(long long columns, int Z) {
+  auto blocks = [&](int zc) { return columns * ((Z + zc - 1) / zc); };
+  int zc = Z;
+  while (zc > 8 && blocks(zc) < 4 * 3 * 152) zc = (zc + 1) / 2;
+  while (zc > 1 && blocks(zc) < 152) zc = (zc + 1) / 2;
+  return zc;
+}
+
 bool cnn_shape_ok(int X, int Y, int Z);
-cudaError_t cnn_pack(const CnnBuffers& w, cudaStream_t s);
+// layer 4 is packed for the kernel that follows: k_conv_out, or k_conv_out_mma in a training step
+cudaError_t cnn_pack(const CnnBuffers& w, bool training, cudaStream_t s);
 // ascale = A = 1/(pi gamma)^2, the fixed output scale
 cudaError_t cnn_forward(const CnnBuffers& w, const float* ubar, float* u0, const float* utrue, int X, int Y, int Z,
                         int B, double ascale, cudaStream_t s);
