@@ -1378,7 +1378,11 @@ ad_status capture_group(ad_ctx* ctx, BatchedGroup& gr, cudaStream_t s, cudaGraph
 // block sizes go to a launch of their own. 2D groups take no part in the y
 // stages. The fields' dot reductions and scalar recurrences stay per group;
 // the count of finished fields and the loop condition span all groups
-// (MultiState).
+// (MultiState). The launches of one stage work on different groups and run
+// side by side, the largest first; one after the other, each waited for the last
+// blocks of the one before. Dot passes of many blocks end in k_finish launches
+// here too, one per group. 48 uneven fields of 19 shapes, 4 to 11 launches a
+// stage: 262 Mpoints/s one after the other, 287 side by side, 312 with k_finish.
 
 int stage_slot(int kind) {
   switch (kind) {
@@ -1391,10 +1395,11 @@ int stage_slot(int kind) {
 }
 
 struct MultiLaunch {
-  int kind = 0, E = 0, blocks = 0, threads = 0, ngroups = 0;
+  int stage = 0, kind = 0, E = 0, blocks = 0, threads = 0, ngroups = 0;
   size_t smem = 0;
   const void* args = nullptr;          // device PassArgs<float>[ngroups]
   const int* start = nullptr;          // device int[ngroups + 1]
+  std::vector<LaunchRec> finish;       // groups whose dots are finished by a launch of their own (PassArgs::defer)
 };
 
 // Lines the groups' recorded launches up by stage and uploads one launch per
@@ -1420,6 +1425,7 @@ ad_status merge_multi(ad_ctx* ctx, BatchedEntry& be, std::vector<std::vector<Lau
     for (auto& byE : st.second) {
       const auto& rs = byE.second;
       MultiLaunch m;
+      m.stage = st.first;
       m.kind = rs[0]->kind;
       m.E = byE.first.first;
       m.ngroups = (int)rs.size();
@@ -1431,12 +1437,15 @@ ad_status merge_multi(ad_ctx* ctx, BatchedEntry& be, std::vector<std::vector<Lau
         a.vgy = (int)rs[g]->grid.y;
         a.vbd = rs[g]->threads;
         a.ms = ms;
-        a.defer = 0;
         if (a.clear_cond) {
           a.clear_cond = (first_clear && !cleared) ? 1 : 0;
           cleared = true;
         }
         args[g] = a;
+        if (a.defer) {
+          m.finish.push_back(*rs[g]);
+          m.finish.back().af = a;
+        }
         start[g + 1] = start[g] + (int)(rs[g]->grid.x * rs[g]->grid.y);
         m.threads = std::max(m.threads, rs[g]->threads);
         m.smem = std::max(m.smem, rs[g]->smem);
@@ -1457,17 +1466,51 @@ ad_status merge_multi(ad_ctx* ctx, BatchedEntry& be, std::vector<std::vector<Lau
       m.start = (const int*)ds;
       out.push_back(m);
     }
+    // the largest first: what is left at the end of a stage is then small
+    auto work = [](const MultiLaunch& m) { return (long long)m.blocks * m.threads * m.E; };
+    std::sort(out.end() - (long)st.second.size(), out.end(),
+              [&](const MultiLaunch& a, const MultiLaunch& b) { return work(a) > work(b); });
   }
   return AD_OK;
 }
 
-cudaError_t issue_multi(const std::vector<MultiLaunch>& ml, cudaStream_t s) {
-  for (const MultiLaunch& m : ml) {
-    const cudaError_t e = launch_multi<float>(m.kind, m.E, m.blocks, m.threads, m.smem, s,
-                                              static_cast<const PassArgs<float>*>(m.args), m.start, m.ngroups);
-    if (e != cudaSuccess) return e;
+// The most launches that one stage of `ml` has.
+size_t widest_stage(const std::vector<MultiLaunch>& ml) {
+  size_t most = 0, n = 0;
+  for (size_t i = 0; i < ml.size(); ++i) {
+    n = i > 0 && ml[i].stage == ml[i - 1].stage ? n + 1 : 1;
+    most = std::max(most, n);
   }
-  return cudaSuccess;
+  return most;
+}
+
+// Captures the launches on `s`, those of a stage after the first on branch
+// streams first_branch, first_branch + 1, .. that leave `s` before the stage
+// and join it again after. A branch stream belongs to one capture only.
+cudaError_t issue_multi(ad_ctx* ctx, const std::vector<MultiLaunch>& ml, cudaStream_t s, size_t first_branch) {
+  cudaError_t e = cudaSuccess;
+  for (size_t i = 0, j = 0; i < ml.size() && e == cudaSuccess; i = j) {
+    for (j = i; j < ml.size() && ml[j].stage == ml[i].stage; ++j) {}
+    cudaEvent_t fork = ctx->events[2 * first_branch];
+    if (j - i > 1) e = cudaEventRecord(fork, s);
+    for (size_t k = i; k < j && e == cudaSuccess; ++k) {
+      const MultiLaunch& m = ml[k];
+      const size_t br = first_branch + k - i - 1;
+      cudaStream_t bs = k == i ? s : ctx->branches[br];
+      if (k > i) e = cudaStreamWaitEvent(bs, fork, 0);
+      if (e == cudaSuccess)
+        e = launch_multi<float>(m.kind, m.E, m.blocks, m.threads, m.smem, bs,
+                                static_cast<const PassArgs<float>*>(m.args), m.start, m.ngroups);
+      for (size_t q = 0; q < m.finish.size() && e == cudaSuccess; ++q) {
+        const LaunchRec& r = m.finish[q];
+        e = launch_finish<float>(r.af, (int)r.grid.x, (int)r.grid.y, r.threads, bs);
+      }
+      if (k > i && e == cudaSuccess) e = cudaEventRecord(ctx->events[2 * br + 1], bs);
+    }
+    for (size_t k = i + 1; k < j && e == cudaSuccess; ++k)
+      e = cudaStreamWaitEvent(s, ctx->events[2 * (first_branch + k - i - 1) + 1], 0);
+  }
+  return e;
 }
 
 // Float32 physical-space Van Cittert, SD, CG and BiCGSTAB without a
@@ -1550,6 +1593,8 @@ ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* 
   std::vector<MultiLaunch> minit, mbody;
   if (st == AD_OK) st = merge_multi(ctx, be, rinit, ms, false, minit);
   if (st == AD_OK) st = merge_multi(ctx, be, rbody, ms, true, mbody);
+  const size_t winit = widest_stage(minit);
+  if (st == AD_OK) st = ensure_streams(ctx, winit + widest_stage(mbody));
   if (st != AD_OK) { cudaGraphDestroy(g); return st; }
   e = cudaStreamBeginCaptureToGraph(ctx->cap, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) { cudaGraphDestroy(g); return cuda_fail(ctx, e, "cudaStreamBeginCaptureToGraph"); }
@@ -1564,7 +1609,7 @@ ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* 
     if (e == cudaSuccess) e = launch_reset_state(gr.p->st, (int)gr.fields.size(), ctx->cap);
     if (e != cudaSuccess) st = cuda_fail(ctx, e, "multi-group gather");
   }
-  if (st == AD_OK && (e = issue_multi(minit, ctx->cap)) != cudaSuccess) st = cuda_fail(ctx, e, "multi-group init");
+  if (st == AD_OK && (e = issue_multi(ctx, minit, ctx->cap, 0)) != cudaSuccess) st = cuda_fail(ctx, e, "multi-group init");
   if (st == AD_OK) {
     cudaStreamCaptureStatus cs;
     cudaGraph_t cg = nullptr;
@@ -1585,7 +1630,7 @@ ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* 
       e = cudaStreamBeginCaptureToGraph(ctx->cap2, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                         cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      const cudaError_t eb = issue_multi(mbody, ctx->cap2);
+      const cudaError_t eb = issue_multi(ctx, mbody, ctx->cap2, winit);
       cudaGraph_t bg = nullptr;
       e = cudaStreamEndCapture(ctx->cap2, &bg);
       if (eb != cudaSuccess) e = eb;
@@ -1617,8 +1662,13 @@ ad_status build_batched_multi(ad_ctx* ctx, BatchedEntry& be, const void* const* 
   be.g = g;
   be.exec = exec;
   be.multi = true;
-  be.m_init = (int)minit.size() + (int)G + (int)small.size();
-  be.m_body = (int)mbody.size();
+  auto launches_of = [](const std::vector<MultiLaunch>& ml) {
+    int n = 0;
+    for (const MultiLaunch& m : ml) n += 1 + (int)m.finish.size();
+    return n;
+  };
+  be.m_init = launches_of(minit) + (int)G + (int)small.size();
+  be.m_body = launches_of(mbody);
   be.m_fin = nfin;
   return AD_OK;
 }
