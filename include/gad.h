@@ -241,8 +241,9 @@ ad_status ad_guess_time_conv(ad_ctx* ctx, const ad_grid* grid, int batch, int re
  * for every pass of one iteration of `method` it times each admissible tile
  * width (32-256 threads per block, <= 100 KB shared memory) with CUDA events
  * on the context's internal buffers and keeps the fastest; later solves on
- * that plan use the tuned tiles (cached graphs are rebuilt). Blocks the host
- * while timing. `enable_for_batched` != 0 makes ad_deconvolve_batched tune
+ * that plan use the tuned tiles (cached graphs are rebuilt). Where a solve by
+ * `method` is one kernel (few small 2D fields, see above) there is nothing to
+ * tune and the call does nothing. Blocks the host while timing. `enable_for_batched` != 0 makes ad_deconvolve_batched tune
  * every plan it creates (0 turns that off); `grid` may be NULL to set only
  * this flag. No counterpart in the paper. */
 ad_status ad_autotune(ad_ctx* ctx, const ad_grid* grid, int batch, ad_method method, int enable_for_batched);

@@ -1105,6 +1105,8 @@ double time_kind(ad_ctx* ctx, Plan* p, int method, int kind, int dots, int reps)
 }
 
 ad_status autotune_plan(ad_ctx* ctx, Plan* p, int method, int reps) {
+  // one kernel per solve: no tiles to tune, and those of the plan's other solves stay as they are
+  if (solves_in_cluster(p, method_spectral(method), method_precond(method))) return AD_OK;
   ad_status s;
   if ((s = ensure_vectors(ctx, p)) != AD_OK || (s = ensure_hist(ctx, p, 1)) != AD_OK) return s;
   if (!p->Uscratch && (s = dmalloc(ctx, p, &p->Uscratch, (size_t)p->P * p->batch * (p->f64 ? 8 : 4))) != AD_OK)
