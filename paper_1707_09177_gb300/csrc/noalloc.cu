@@ -107,11 +107,10 @@ struct StaticPass {
   dim3 grid;
 };
 
-// The same plan and tile shape as the context-owning entry points build
-// (plan.h), so the pass kernels take the same code paths.
-bool plan_s(int L, int slots, int div, long long nseq, bool transposed, size_t cs, const void* tab,
-            const void* tab_inv, StaticPass& pc) {
-  if (!choose_pass(L, slots, div, nseq, transposed, cs, pc.t)) return false;
+// The plan of a pass whose tile is chosen. The tiles are those of the passes
+// that ad_filter launches (grid_tiles, plan.h), so the kernels take the same
+// code paths; ad_filter's one-kernel path for few small 2D fields is not taken.
+bool plan_s(int L, size_t cs, const void* tab, const void* tab_inv, StaticPass& pc) {
   const int E = plan_E(L, pc.t.E, cs);
   if (!make_fft(L, E, tab, pc.fft)) return false;
   return !tab_inv || make_fft(L, E, tab_inv, pc.fft_inv, true);
@@ -157,15 +156,22 @@ ad_status run_static(const ad_grid* g, const void* in, void* out, int batch, cud
   void* S1 = b + tabs;
   void* S2 = g->ndim == 3 ? (void*)(b + tabs + sb) : nullptr;
 
-  StaticPass xf, fl, yf;
+  StaticPass xf, xi, fl, yf;
   const int nseq = g->ndim == 3 ? kxn * ny : kxn;
-  bool ok = plan_s(M, M + 1, pow2_part(ny), (long long)ny * nz, true, cs, tpx_d, nullptr, xf);
-  ok = ok && plan_s(Lf, Lf, 0, nseq, false, cs, tpf_d, tpfi_d, fl);
-  if (g->ndim == 3) ok = ok && plan_s(ny, ny, pow2_part(nz), (long long)kxn * nz, true, cs, tpy_d, nullptr, yf);
+  GridTiles gt;
+  if (!grid_tiles(nx, ny, nz, batch, cs, gt)) return AD_ERR_ARG;
+  xf.t = gt.xf;
+  xi.t = gt.xi_nodots.E == gt.xf.E ? gt.xi_nodots : gt.xf;   // one x plan in the scratch
+  fl.t = gt.fl_nodots;
+  yf.t = gt.y;
+  bool ok = plan_s(M, cs, tpx_d, nullptr, xf) && plan_s(M, cs, tpx_d, nullptr, xi) && plan_s(Lf, cs, tpf_d, tpfi_d, fl);
+  if (g->ndim == 3) ok = ok && plan_s(ny, cs, tpy_d, nullptr, yf);
   if (!ok) return AD_ERR_ARG;
-  xf.rcp_a = 1.0f / (float)(nx / 4);
-  xf.rcp_b = 1.0f / (float)(M / 2 + 1);
-  xf.grid = dim3(ny * nz / xf.t.W, batch);
+  for (StaticPass* x : {&xf, &xi}) {
+    x->rcp_a = 1.0f / (float)(nx / 4);
+    x->rcp_b = 1.0f / (float)(M / 2 + 1);
+    x->grid = dim3(ny * nz / x->t.W, batch);
+  }
   fl.grid = dim3((nseq + fl.t.W - 1) / fl.t.W, batch);
   if (g->ndim == 3) yf.grid = dim3(kxn * (nz / yf.t.W), batch);
 
@@ -200,7 +206,7 @@ ad_status run_static(const ad_grid* g, const void* in, void* out, int batch, cud
   if (launch(PK_FILT, fl) != cudaSuccess) return AD_ERR_CUDA;
   if (g->ndim == 3 && launch(PK_YINV, yf) != cudaSuccess) return AD_ERR_CUDA;
   a.op = XI_STORE; a.O1 = static_cast<T*>(out);
-  if (launch(PK_XINV, xf) != cudaSuccess) return AD_ERR_CUDA;
+  if (launch(PK_XINV, xi) != cudaSuccess) return AD_ERR_CUDA;
   return AD_OK;
 }
 
