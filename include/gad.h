@@ -32,10 +32,10 @@
  *   - A context is not thread safe; use one context per host thread.
  *   - A field's result does not depend on the other fields of its call. On 2D
  *     grids of up to 256^2 points (float32) or 128^2 (float64) it may differ in
- *     its last bits between calls of few and of many such fields: up to as
- *     many as the GPU runs at once (14 of the largest) are filtered, and solved
- *     by Algorithms 1-4 in physical space, by one kernel that adds in another
- *     order. Elsewhere a field's result is the same bits in every batch.
+ *     its last bits between calls of few and of many such fields: up to 14 (28
+ *     on grids of up to 128^2 points in float32, more where the GPU runs more
+ *     of them at once) are filtered, and solved by Algorithms 1-4 in physical
+ *     space, by one kernel that adds in another order. Elsewhere a field's result is the same bits in every batch.
  */
 #ifndef GAD_H
 #define GAD_H

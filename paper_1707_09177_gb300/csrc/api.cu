@@ -393,15 +393,10 @@ ad_status get_plan(ad_ctx* ctx, const ad_grid* g, int batch, Plan** out) {
     p->sn.rcp_a = 1.0f / (float)(p->nx / 4);
     p->sn.grid = dim3((unsigned)(tiles * (nmarch / chunk)), batch);
   }
-  // clusters only while every field's runs at once (14 of 16 CTAs): a cluster is
-  // a chain of latencies, and a second round of them doubles it, where the pass
-  // kernels hardly notice more fields. Cluster / pass kernels, us: 3 BiCGSTAB
-  // passes on 256^2 float32, 1 field 197 / 334, 14 223 / 351, 16 356 / 326, 40
-  // 545 / 414; on 64^2 float64 1 field 329 / 428, 14 343 / 431, 16 604 / 431, 128
-  // 2660 / 825; filter of 128^2 float64, 1 field 37 / 39, 40 134 / 103
+  // clusters only while the fields' run in cluster_rounds (plan.h) rounds
   if (cluster_shape(p->nx, p->ny, p->nz, cs, p->cl) &&
-      batch <= (p->f64 ? cluster_room<double>(p->cl.csize, p->cl.threads, p->cl.smem)
-                       : cluster_room<float>(p->cl.csize, p->cl.threads, p->cl.smem))) {
+      batch <= cluster_rounds(p->P, cs) * (p->f64 ? cluster_room<double>(p->cl.csize, p->cl.threads, p->cl.smem)
+                                                  : cluster_room<float>(p->cl.csize, p->cl.threads, p->cl.smem))) {
     const void *tx8 = nullptr, *tl8 = nullptr;
     if ((s = get_plan_table(ctx, M, kClusterE, false, p->f64, &tx8)) != AD_OK ||
         (s = get_plan_table(ctx, Lf, kClusterE, false, p->f64, &tl8)) != AD_OK) {
@@ -879,9 +874,8 @@ ad_status enqueue_finish(ad_ctx* ctx, Plan* p, cudaStream_t s, const SolveIO& io
   return io.want_true ? enqueue_true<T>(ctx, p, s, io, c, nl) : AD_OK;
 }
 
-// A solve that one cluster per field runs in one launch: up to as many fields of
-// a small grid as run at once (get_plan), the physical-space methods without a
-// preconditioner. The clusters add the dots in another order than the pass
+// A solve that one cluster per field runs in one launch: a few fields of a small
+// grid (get_plan), the physical-space methods without a preconditioner. The clusters add the dots in another order than the pass
 // kernels that take the larger batches (and their transforms have other
 // radices), so a small field's result is the same bits alone and in a batch only
 // as long as both are on one side of that limit.

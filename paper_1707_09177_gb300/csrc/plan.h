@@ -350,6 +350,15 @@ struct ClusterShape {
 constexpr size_t kClusterSmem = 224 * 1024;   // dynamic shared memory a CTA may take
 constexpr int kClusterE = 24;                 // element count whose plans have radices of at most 8
 
+// Rounds of clusters that a batch may take (the GPU holds 14 of 16 CTAs at a
+// time); more fields take the pass kernels. A cluster is a chain of latencies
+// and a further round of them as long again, where the pass kernels hardly
+// notice more fields. 3 BiCGSTAB passes, cluster / pass kernels, us: 256^2
+// float32 1 field 197 / 334, 14 223 / 351, 16 356 / 326, 40 545 / 414; 128^2
+// float32 16 to 28 fields 290 / 400, 40 400 / 403; 64^2 float64 14 fields
+// 343 / 431, 16 604 / 431, 128 2660 / 825.
+inline int cluster_rounds(long long points, size_t csize) { return csize == 8 && points <= 128 * 128 ? 2 : 1; }
+
 // False when the grid is not one for a cluster: it takes the pass kernels.
 // Measured per pass of a single field, cluster against pass kernels: CG float32
 // 256^2 18 against 40 us; Van Cittert float64 128^2 36 against 53 us (the

@@ -35,6 +35,17 @@ def test_solves_of_few_and_many_small_fields(gad, method, dtype):
             assert _rel(res.u[i].double().cpu().numpy(), r) < tol, (n, i)
 
 
+def test_a_second_round_only_where_it_is_short(gad):
+    """20 fields are two rounds of clusters: still one launch on 128^2 float32,
+    the pass kernels on 192^2 float32 and 128^2 float64."""
+    import torch
+    for shape, dtype, one in (((128, 128), torch.float32, True), ((192, 192), torch.float32, False),
+                              ((128, 128), torch.float64, False)):
+        t = torch.rand((20,) + shape, device="cuda", dtype=dtype)
+        gad.deconvolve(t, 0.2, method="cg", tol=0.0, maxit=2, ndim=2)
+        assert (gad.last_launch_count() == 1) == one, (shape, dtype)
+
+
 @pytest.mark.parametrize("dtype,tol", [(np.float32, 3e-6), (np.float64, 1e-13)])
 def test_filter_and_closure_of_few_and_many_small_fields(gad, dtype, tol):
     import torch
