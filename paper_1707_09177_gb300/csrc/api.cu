@@ -1832,7 +1832,9 @@ ad_status ad_time_pass(ad_ctx* ctx, const ad_grid* grid, int batch, ad_method me
   cudaEventDestroy(e1);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "ad_time_pass");
   if (ms_per_launch) *ms_per_launch = (double)ms / reps;
-  ctx->launches = (long long)(reps + 1) * (long long)(last - first);
+  long long per = 0;                                 // a deferred dot pass is two launches
+  for (size_t i = first; i < last; ++i) per += 1 + (rec[i].f64 ? rec[i].ad.defer : rec[i].af.defer);
+  ctx->launches = (long long)(reps + 1) * per;
   return AD_OK;
 }
 
