@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(128, 3) k_conv_1ch(const float* __restrict__ S
   for (int i = threadIdx.x; i < TAPS * C; i += blockDim.x) w[i] = W[i];
   __syncthreads();
   const float scale = BWD ? 1.f : (float)(1.0 / sqrt(fmax(sumsq[b] / (double)P, 1e-300)));
-  const long long groups = P >> 2;                   // a multiple of 32: X is (and Y, Z are even), or Y Z 8 is
+  const long long groups = P >> 2;                   // not always a multiple of 32: the last warp's lanes are guarded
   for (long long pg0 = blockIdx.x * (long long)blockDim.x + threadIdx.x - lane; pg0 < groups;
        pg0 += (long long)gridDim.x * blockDim.x) {
     const long long pg = min(pg0 + lane, groups - 1);

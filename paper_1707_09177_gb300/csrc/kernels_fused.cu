@@ -1,4 +1,4 @@
-// Float32 pass kernels compiled for one transform length with a factor 3 each,
+// Float32 pass kernels compiled for one transform length 2^a 3 or 2^a 9 each,
 // at 12 elements per thread (fused radices, plan.h): constant strides instead
 // of the general stages' float quotients, no spills. Two translation units
 // (GAD_LONG 0: up to 192, 1: longer) that compile in parallel.

@@ -105,10 +105,15 @@ constexpr RadixSeq fused_radices(int L, int E) {
 }
 
 // Lengths of those plans, at 12 elements per thread: 64 registers and 4 blocks
-// per SM with nothing spilled (the filter pass at 24 elements spills 900 bytes
-// per thread at 80 registers). A transposed tile of more than 768 elements per
-// row would hold fewer than the four rows of a 32-byte sector in 256 threads
-// and keeps 24 elements.
+// per SM, with nothing spilled in the kernels compiled for 2^a 3 and 2^a 9
+// (kernels_fused.cu) and 64 bytes in the filter pass of the general stages that
+// the other lengths (108, 162, 216, 324, 432, 648, 864, ..) run; at 24 elements
+// it spills 900 bytes per thread at 80 registers. The general stages gain from
+// the fewer stages too, 24 separate against 12 fused elements, us: filter of
+// 216^3 x 3 783 / 545, 324^3 x 3 2539 / 2009, 864^2 x 8 142 / 88, 1728^2 x 8
+// 471 / 383. A transposed tile of more than 768 elements per row would hold
+// fewer than the four rows of a 32-byte sector in 256 threads and keeps 24
+// elements.
 constexpr bool fused_length(int L) { return L % 3 == 0 && L >= 36 && L <= 2304 && fused_radices(L, 12).n > 0; }
 
 // Key of a plan: its element count, odd for the fused radices.
@@ -363,7 +368,10 @@ inline int cluster_rounds(long long points, size_t csize) { return csize == 8 &&
 // Measured per pass of a single field, cluster against pass kernels: CG float32
 // 256^2 18 against 40 us; Van Cittert float64 128^2 36 against 53 us (the
 // float64 rate of 16 SMs, two lanes per clock each, is the larger part of it and
-// grows with the points). 3D fields have four more transposing steps through
+// grows with the points). The float64 limit lies where powers of two stop
+// gaining (10 CG passes, us: 128^2 545 / 685, 128 x 256 766 / 706, 256^2 1324 /
+// 719); float32 gains up to about 400^2 (256^2 265 / 508, 288^2 320 / 422, 384^2
+// 401 / 459), its limit is where the gain is largest. 3D fields have four more transposing steps through
 // shared memory and gain nothing (64^3 float32 CG: 53 against 50 us).
 constexpr long long kClusterPoints32 = 256 * 256, kClusterPoints64 = 128 * 128;
 
