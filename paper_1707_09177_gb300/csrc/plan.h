@@ -245,8 +245,11 @@ inline bool choose_tile(int L, int E, int slots, int div, size_t csize, TileShap
 // field where it has dots, of all its fields where it has none. Two blocks per
 // SM for the launches without dots: with one, 32 fields of 192^2 float64 filter
 // in 259 us, with two in 198, with four 64^3 float32 x 4 takes 54 against 51 us.
+// Four for float64 powers of two, bound by the float64 rate of the busiest SM
+// (16 fields of 256^2 148 us against 154, four of 64^3 159 against 177); lengths
+// with a factor 3 lose by it there (16 fields of 288^2 270 against 214).
 constexpr int kWantBlocks = 152;
-constexpr int kWantLaunch = 2 * 152;
+inline int want_launch(int L, size_t csize) { return (csize == 16 && L % 3 != 0 ? 4 : 2) * 152; }
 // Complex elements per field below which a pass takes small_E: with the default
 // count less than a third of the GPU's threads would have work. For powers of
 // two (float64) a quarter of that: one 64^3 field (135,168 elements) filters in
@@ -300,7 +303,7 @@ inline bool choose_pass(int L, int slots, int div, long long nseq, bool transpos
   }
   auto enough = [&](int W) {
     const long long n = (nseq + W - 1) / W;
-    return batch > 0 ? n * batch >= kWantLaunch : n >= kWantBlocks;
+    return batch > 0 ? n * batch >= want_launch(L, csize) : n >= kWantBlocks;
   };
   int rad[kMaxStages];
   int E = E0;

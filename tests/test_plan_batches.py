@@ -87,3 +87,17 @@ def test_few_elements_per_thread_only_where_a_batch_gains_too(tiles):
                 assert cs == 16 and kx * grid[1] * grid[2] < 152 * 16 * 16, (grid, cs, k)
     assert tiles[(512, 512, 1), 8, 16]["fl"][0] == tiles[(64, 64, 64), 8, 1]["fl"][0] == 16
     assert tiles[(256, 256, 1), 16, 1]["fl"][0] == 4 and tiles[(64, 64, 64), 16, 1]["fl"][0] == 16
+
+
+def test_blocks_wanted_of_a_launch_without_dots(tiles):
+    """A launch keeps a wide tile only where that gives two blocks per SM, four
+    for float64 powers of two."""
+    for (grid, cs, batch), r in tiles.items():
+        nx, ny, nz = grid
+        if not r["ok"]:
+            continue
+        L, seqs = (nz, (nx // 2 + 1) * ny) if nz > 1 else (ny, nx // 2 + 1)
+        E, W, T = r["fl_nodots"][:3]
+        want = 152 * (4 if cs == 16 and L % 3 else 2)
+        assert -(-seqs // W) * batch >= want or W == 1 or T // 2 < 32, (grid, cs, batch, r["fl_nodots"])
+    assert tiles[(64, 64, 64), 16, 3]["fl_nodots"][1] < tiles[(64, 64, 64), 16, 16]["fl_nodots"][1]
