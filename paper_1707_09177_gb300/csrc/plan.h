@@ -255,7 +255,8 @@ inline int want_launch(int L, size_t csize) { return (csize == 16 && L % 3 != 0 
 // two (float64) a quarter of that: one 64^3 field (135,168 elements) filters in
 // 68 us with 4 elements and 111 with 16, but the closure of 32 such velocities
 // takes 6.6 against 6.1 ms; 256^2 (33,024): 39 against 88 us for one, 2.10
-// against 1.93 ms for 256 (2.06 before narrow tiles).
+// against 1.93 ms for 256 (2.06 before narrow tiles); 32^3 (17,408): 49 against
+// 95 us for one, closure of 128 velocities 3.06 against 2.75 ms (2.89 before).
 constexpr long long kSmallElems = 152 * 64 * 16, kSmallElemsPow2 = kSmallElems / 4;
 
 // Row stride of a tile of W rows that is stored or loaded transposed (the W
